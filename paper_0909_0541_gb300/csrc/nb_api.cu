@@ -303,22 +303,6 @@ int nb_grow_queues(nb_ctx *c)
     return alloc_queues(c, want) ? NB_OK : NB_ERR_NOMEM;
 }
 
-// the largest root-cube side over the current tree's systems (synchronising)
-double nb_root_side(nb_ctx *c)
-{
-    double L = 0.0;
-    for (int64_t sy = 0; sy < c->nsys; sy++) {
-        double v = 0.0;
-        if (cudaMemcpy(&v, c->root + 8 * sy + 3, sizeof(double), cudaMemcpyDeviceToHost) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            return 0.0;
-        }
-        if (v > L) L = v;
-    }
-    return L;
-}
-
 static int finish(nb_ctx *c)
 {
     if (cudaGetLastError() != cudaSuccess) return NB_ERR_CUDA;

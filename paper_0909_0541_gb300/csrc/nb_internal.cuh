@@ -311,7 +311,6 @@ int nb_neigh_run(nb_ctx *c, double h, int n_crit, int64_t *off, int32_t *idx, in
 int nb_read_err(nb_ctx *c, unsigned *bits);
 int nb_err_code(unsigned bits);
 int nb_grow_queues(nb_ctx *c);
-double nb_root_side(nb_ctx *c);
 #define CK_RET(call)                                                        \
     do {                                                                    \
         if ((call) != cudaSuccess) {                                        \
