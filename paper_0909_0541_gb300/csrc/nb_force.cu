@@ -34,8 +34,12 @@
 // first and the kernel does not end on one warp finishing a long list.  An
 // item's result does not depend on when it runs, so the order changes
 // timing only.
+#include <cooperative_groups.h>
+
 #include "nb_force.cuh"
 #include "nb_walk.cuh"
+
+namespace cg = cooperative_groups;
 
 #define F_T 256
 
@@ -584,50 +588,129 @@ void nb_launch_walk_force(nb_ctx *c, float eps, float *acc, float *pot, int prec
 }
 
 // ---------------------------------------------------------------- judge
-// FP64 direct sum: one block per target, a deterministic tree reduction.
-__global__ void __launch_bounds__(256)
-k_direct(const double *__restrict__ pos, const float *__restrict__ mass, int64_t n,
-         double eps2, const int64_t *__restrict__ targets, int64_t nt,
-         double *__restrict__ acc, double *__restrict__ pot)
+// FP64 direct sum.  Bound by the FP64 pipe, which takes 16 cycles of an SM
+// for one warp instruction: what counts is the number of FP64 operations per
+// pair and that every SM has an equal share.  A pair takes 18: 3 differences,
+// 3 for r^2 + eps^2, 5 for 1/r from an FP32 seed, 3 for m/r and m/r^3, 4 for
+// the sums; the conversions, which would take the pipe too, are integer
+// instructions.  With sqrt, a division and conversions, 4096 targets x
+// 524,288 sources took 120.3 ms; it takes 71.5 ms so, 0.86 of the pipe's
+// rate (2 lanes per clock and SM).
+//
+// A block takes DJ_R targets (two share a source's loads: 71.5 against 73.6
+// ms with one, 98 with four, whose registers leave too few warps; warps of 8
+// or 32 targets reading the same source: 76 and 87 ms) and its threads stride
+// over the sources.  With few targets the blocks of a cluster share the
+// sources.  The threads' sums are added by shuffles, then over the warps and
+// the cluster's blocks in a fixed order: the result does not depend on
+// timing, and no workspace is needed.
+#define DJ_T 256
+#define DJ_R 2
+
+// FP32 to FP64 by integer instructions (a conversion instruction takes FP64
+// pipe time), exact for normal numbers; the others take the conversion
+__device__ __forceinline__ double widen(float f)
 {
-    __shared__ double red[4][256];
-    for (int64_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int64_t i = targets ? targets[t] : t;
-        const double xi = pos[3 * i], yi = pos[3 * i + 1], zi = pos[3 * i + 2];
-        double ax = 0.0, ay = 0.0, az = 0.0, p = 0.0;
-        for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-            if (j == i) continue;
-            const double dx = pos[3 * j] - xi, dy = pos[3 * j + 1] - yi, dz = pos[3 * j + 2] - zi;
-            const double r2 = dx * dx + dy * dy + dz * dz + eps2;
-            if (r2 == 0.0) continue;
-            const double ri = 1.0 / sqrt(r2);
-            const double m = (double)mass[j];
-            const double mr3 = m * ri * ri * ri;
-            ax += mr3 * dx;
-            ay += mr3 * dy;
-            az += mr3 * dz;
-            p -= m * ri;
-        }
-        red[0][threadIdx.x] = ax;
-        red[1][threadIdx.x] = ay;
-        red[2][threadIdx.x] = az;
-        red[3][threadIdx.x] = p;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (threadIdx.x < o)
-                for (int k = 0; k < 4; k++) red[k][threadIdx.x] += red[k][threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            acc[3 * t] = red[0][0];
-            acc[3 * t + 1] = red[1][0];
-            acc[3 * t + 2] = red[2][0];
-            pot[t] = red[3][0];
-        }
-        __syncthreads();
-    }
+    const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+    return (double)f;
 }
 
+// 1 / sqrt(r2).  The seed y is the FP32 unit's for r2 cut to 24 bits, moved
+// between the formats with integer instructions: a relative error below
+// 2^-21.  With e = 1 - r2 y^2 the series 1/sqrt(1 - e) = 1 + e/2 + 3 e^2/8 +
+// O(e^3) leaves (5/16) e^3 < 2^-61 beside the rounding of its last steps.
+// Outside FP32's normal range (and for non-finite r2) the square root and
+// the division; r2 = 0 (a coincident pair without softening) gives 0, so
+// that it contributes nothing.
+__device__ __forceinline__ double judge_rsqrt(double r2)
+{
+    const unsigned hi = (unsigned)__double2hiint(r2), lo = (unsigned)__double2loint(r2);
+    if (hi - 0x38200000u < 0x0fa00000u) {   // 2^-125 <= r2 < 2^125
+        const float yf = mufu_rsqrt(__uint_as_float(__funnelshift_l(lo, hi - 0x38000000u, 3)));
+        const unsigned b = __float_as_uint(yf);
+        const double y = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+        const double e = __fma_rn(-__dmul_rn(r2, y), y, 1.0);
+        return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
+    }
+    return r2 == 0.0 ? 0.0 : 1.0 / sqrt(r2);
+}
+
+__global__ void __launch_bounds__(DJ_T)
+k_direct(const double *__restrict__ pos, const float *__restrict__ mass, int64_t n,
+         double eps2, const int64_t *__restrict__ targets, int64_t first, int64_t nt,
+         double *__restrict__ acc, double *__restrict__ pot)
+{
+    constexpr int WARPS = DJ_T / NB_WARP;
+    __shared__ double part[WARPS][DJ_R][4];
+    __shared__ double sum[DJ_R][4];
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t t0 = first + (int64_t)(blockIdx.x / C) * DJ_R;
+    double x[DJ_R][3], v[DJ_R][4];
+    int64_t self[DJ_R];
+#pragma unroll
+    for (int r = 0; r < DJ_R; r++) {
+        const int64_t t = t0 + r < nt ? t0 + r : nt - 1;
+        self[r] = targets ? targets[t] : t;
+#pragma unroll
+        for (int k = 0; k < 3; k++) x[r][k] = pos[3 * self[r] + k];
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[r][k] = 0.0;
+    }
+    const int64_t stride = (int64_t)C * DJ_T;
+#pragma unroll 2
+    for (int64_t j = rank * DJ_T + threadIdx.x; j < n; j += stride) {
+        const double xj = pos[3 * j], yj = pos[3 * j + 1], zj = pos[3 * j + 2];
+        const double mj = widen(mass[j]);
+#pragma unroll
+        for (int r = 0; r < DJ_R; r++) {
+            const double dx = xj - x[r][0], dy = yj - x[r][1], dz = zj - x[r][2];
+            const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __fma_rn(dx, dx, eps2)));
+            const double ri = judge_rsqrt(r2);
+            const double mr = (j == self[r] ? 0.0 : mj) * ri;
+            const double w3 = mr * ri * ri;
+            v[r][0] = __fma_rn(w3, dx, v[r][0]);
+            v[r][1] = __fma_rn(w3, dy, v[r][1]);
+            v[r][2] = __fma_rn(w3, dz, v[r][2]);
+            v[r][3] -= mr;
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < NB_WARP; o <<= 1)
+#pragma unroll
+        for (int r = 0; r < DJ_R; r++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) v[r][k] += __shfl_xor_sync(0xffffffffu, v[r][k], o);
+    if (lane == 0)
+#pragma unroll
+        for (int r = 0; r < DJ_R; r++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) part[w][r][k] = v[r][k];
+    __syncthreads();
+    const int r = threadIdx.x >> 2, k = threadIdx.x & 3;
+    if (r < DJ_R) {
+        double s = part[0][r][k];
+        for (int p = 1; p < WARPS; p++) s += part[p][r][k];
+        sum[r][k] = s;
+    }
+    cl.sync();
+    if (rank == 0 && r < DJ_R && t0 + r < nt) {
+        double s = sum[r][k];
+        for (int p = 1; p < C; p++) s += *cl.map_shared_rank(&sum[r][k], p);
+        if (k < 3) acc[3 * (t0 + r) + k] = s;
+        else pot[t0 + r] = s;
+    }
+    cl.sync();   // every block's sums stay until rank 0 has read them
+}
+
+// Clusters of as many blocks (up to the portable 8) as give every SM 24, so
+// that the last round of blocks is a small part of the work (4096 targets:
+// 74.1 ms with 13 blocks per SM, 71.5 with 27), while each block keeps 2048
+// sources (500 targets, 3000 sources: 73 us with one block per target pair,
+// 119 with eight).
 int nb_launch_direct(const double *pos, const float *mass, int64_t n, double eps,
                      const int64_t *targets, int64_t nt, double *acc, double *pot,
                      cudaStream_t s)
@@ -636,7 +719,26 @@ int nb_launch_direct(const double *pos, const float *mass, int64_t n, double eps
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t g = nt < (int64_t)sms * 8 ? nt : (int64_t)sms * 8;
-    k_direct<<<(int)g, 256, 0, s>>>(pos, mass, n, eps * eps, targets, nt, acc, pot);
+    const int64_t tb = (nt + DJ_R - 1) / DJ_R;
+    int C = 1;
+    while (C < 8 && tb * C < 24 * (int64_t)sms && n >= 2048 * (int64_t)(2 * C)) C *= 2;
+    const int64_t max_tb = (int64_t)INT32_MAX / C;
+    // (more target blocks than a grid holds: several launches)
+    for (int64_t done = 0; done < tb; done += max_tb) {
+        const int64_t left = tb - done;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((left < max_tb ? left : max_tb) * C));
+        cfg.blockDim = dim3(DJ_T);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, k_direct, pos, mass, n, eps * eps, targets, done * DJ_R, nt,
+                               acc, pot) != cudaSuccess)
+            return -1;
+    }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
