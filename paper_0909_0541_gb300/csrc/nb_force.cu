@@ -237,6 +237,7 @@ k_item_hist(const int32_t *__restrict__ items, const int32_t *__restrict__ gcoun
             const int32_t *__restrict__ glen, const long long *__restrict__ cnt,
             int64_t max_items, int32_t *__restrict__ bkt)
 {
+    nb_grid_wait();
     __shared__ int32_t h[NB_IBKT];
     if (threadIdx.x < NB_IBKT) h[threadIdx.x] = 0;
     __syncthreads();
@@ -254,6 +255,7 @@ k_item_order(const int32_t *__restrict__ items, const int32_t *__restrict__ gcou
              const int32_t *__restrict__ glen, long long *__restrict__ cnt, int64_t max_items,
              int32_t *__restrict__ bkt, int32_t *__restrict__ order, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     static_assert(NB_IBKT <= 256, "one bucket per thread");
     __shared__ int32_t start[NB_IBKT];
     {
@@ -297,6 +299,7 @@ k_force(const int32_t *__restrict__ items, const int32_t *__restrict__ order,
         float *__restrict__ acc, float *__restrict__ pot, unsigned *__restrict__ err,
         int64_t max_items)
 {
+    nb_grid_wait();
     __shared__ float4 tiles[BT / NB_WARP][QUAD ? TILE * 5 / 2
                                                : (TILE > F_TILE_STREAMS ? TILE : F_TILE_STREAMS)];
     const unsigned FULL = 0xffffffffu;
@@ -361,10 +364,10 @@ static void launch_force_t(nb_ctx *c, float eps2, float *acc, float *pot)
                                                       k_force<MODE, GUARD, TILE, BT, QUAD>, BT, 0);
         if (blocks < 1) blocks = 1;
     }
-    k_force<MODE, GUARD, TILE, BT, QUAD><<<c->num_sms * blocks, BT, 0, c->stream>>>(
-        c->items, c->item_order, c->gfirst, c->gcount, c->glen, c->gbox, c->p_hi, c->p_lo, c->perm,
-        c->list_xm, c->list_q, c->list_cap, c->list_alloc, c->n, c->cnt, eps2, acc, pot, c->err,
-        c->max_items);
+    nb_launch(k_force<MODE, GUARD, TILE, BT, QUAD>, c->num_sms * blocks, BT, 0, nb_queue(c),
+              c->items, c->item_order, c->gfirst, c->gcount, c->glen, c->gbox, c->p_hi, c->p_lo,
+              c->perm, c->list_xm, c->list_q, c->list_cap, c->list_alloc, c->n, c->cnt, eps2, acc,
+              pot, c->err, c->max_items);
     nb_launched(c, QUAD ? "k_force (quadrupole)" : "k_force");
 }
 
@@ -390,11 +393,11 @@ void nb_launch_forces(nb_ctx *c, float eps, float *acc, float *pot, int precisio
     cudaMemsetAsync(&c->cnt[CNT_FORCE_Q], 0, sizeof(long long), c->stream);
     cudaMemsetAsync(c->item_bkt, 0, sizeof(int32_t) * 2 * NB_IBKT, c->stream);
     const int ig = c->num_sms * 2;
-    k_item_hist<<<ig, 256, 0, c->stream>>>(c->items, c->gcount, c->glen, c->cnt, c->max_items,
-                                           c->item_bkt);
+    nb_launch(k_item_hist, ig, 256, 0, nb_queue(c), c->items, c->gcount, c->glen, c->cnt,
+              c->max_items, c->item_bkt);
     nb_launched(c, "k_item_hist");
-    k_item_order<<<ig, 256, 0, c->stream>>>(c->items, c->gcount, c->glen, c->cnt, c->max_items,
-                                            c->item_bkt, c->item_order, c->err);
+    nb_launch(k_item_order, ig, 256, 0, nb_queue(c), c->items, c->gcount, c->glen, c->cnt,
+              c->max_items, c->item_bkt, c->item_order, c->err);
     nb_launched(c, "k_item_order");
     const float eps2 = eps * eps;
     const bool guard = !(eps2 >= FLT_MIN);
@@ -461,6 +464,7 @@ k_walk_force(const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ pid2b
              const int32_t *__restrict__ perm, int64_t n, float eps2, float *__restrict__ acc,
              float *__restrict__ pot, int64_t max_items, int32_t *__restrict__ gready)
 {
+    nb_grid_wait();
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -559,12 +563,12 @@ static void launch_walk_force_t(nb_ctx *c, float eps2, float *acc, float *pot)
     }
     // one pair of frontier queues per warp: no more warps than the queues hold
     const int blocks = c->walk_warps / OV_WARPS;
-    k_walk_force<MODE, GUARD><<<blocks > 0 ? blocks : 1, OV_T, 0, c->stream>>>(
-        c->wrec, c->pid2bfs, c->gnode, c->gcount, c->gbox, c->cnt, c->glen, c->gcells,
-        c->list_id, c->list_xm, c->list_cap, c->list_alloc, c->wq, c->wq_cap, c->err, c->root,
-        c->n_depth, c->gfirst, c->nsys > 1 ? c->sys_sorted : nullptr,
-        c->nsys > 1 ? c->sys_root : nullptr, c->items, c->p_hi, c->p_lo, c->perm, c->n, eps2,
-        acc, pot, c->max_items, c->gready);
+    nb_launch(k_walk_force<MODE, GUARD>, blocks > 0 ? blocks : 1, OV_T, 0, nb_queue(c), c->wrec,
+              c->pid2bfs, c->gnode, c->gcount, c->gbox, c->cnt, c->glen, c->gcells, c->list_id,
+              c->list_xm, c->list_cap, c->list_alloc, c->wq, c->wq_cap, c->err, c->root,
+              c->n_depth, c->gfirst, c->nsys > 1 ? c->sys_sorted : nullptr,
+              c->nsys > 1 ? c->sys_root : nullptr, c->items, c->p_hi, c->p_lo, c->perm, c->n, eps2,
+              acc, pot, c->max_items, c->gready);
     nb_launched(c, "k_walk_force");
 }
 

@@ -231,6 +231,7 @@ k_walk_force(const int32_t *__restrict__ items, const nb_wrec *__restrict__ wrec
              float *__restrict__ pot, int64_t n, int64_t max_items,
              const int32_t *__restrict__ sys_sorted, const int32_t *__restrict__ sys_root)
 {
+    nb_grid_wait();
     __shared__ float4 bufs[FW_WARPS][FW_BUF];
     __shared__ int32_t sq[FW_WARPS][2 * WQ_SMEM];
     const unsigned FULL = 0xffffffffu;
@@ -290,10 +291,10 @@ static void launch_fused(nb_ctx *c, float eps2, float *acc, float *pot)
     int grid = c->num_sms * blocks;
     if ((int64_t)grid * FW_WARPS > c->walk_warps) grid = c->walk_warps / FW_WARPS;
     if (grid < 1) grid = 1;
-    k_walk_force<MODE, GUARD><<<grid, FW_T, 0, c->stream>>>(
-        c->items, c->wrec, c->pid2bfs, c->gnode, c->gfirst, c->gcount, c->gbox, c->p_hi, c->p_lo,
-        c->perm, c->cnt, c->wq, c->wq_cap, c->err, eps2, acc, pot, c->n, c->max_items,
-        c->nsys > 1 ? c->sys_sorted : nullptr, c->nsys > 1 ? c->sys_root : nullptr);
+    nb_launch(k_walk_force<MODE, GUARD>, grid, FW_T, 0, nb_queue(c), c->items, c->wrec, c->pid2bfs,
+              c->gnode, c->gfirst, c->gcount, c->gbox, c->p_hi, c->p_lo, c->perm, c->cnt, c->wq,
+              c->wq_cap, c->err, eps2, acc, pot, c->n, c->max_items,
+              c->nsys > 1 ? c->sys_sorted : nullptr, c->nsys > 1 ? c->sys_root : nullptr);
     nb_launched(c, "k_walk_force");
 }
 

@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(MLP_T)
 k_mlp_infer(const float *__restrict__ P, const float *__restrict__ feat,
             const long long *__restrict__ cnt, float *__restrict__ theta, float fallback)
 {
+    nb_grid_wait();
     __shared__ __align__(16) bf16 sbuf[MLP_T / 32][2][16 * MH];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
@@ -279,7 +280,8 @@ void nb_launch_mlp_infer(nb_ctx *c, const float *params, const float *feat, floa
     int blocks = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_mlp_infer, MLP_T, 0);
     if (blocks < 1) blocks = 1;
-    k_mlp_infer<<<c->num_sms * blocks, MLP_T, 0, c->stream>>>(params, feat, c->cnt, theta, fallback);
+    nb_launch(k_mlp_infer, c->num_sms * blocks, MLP_T, 0, nb_queue(c), params, feat, c->cnt, theta,
+              fallback);
     nb_launched(c, "k_mlp_infer");
 }
 

@@ -183,6 +183,7 @@ k_neigh(const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ items,
         const int32_t *__restrict__ sys_sorted, const int32_t *__restrict__ sys_root,
         unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const unsigned FULL = 0xffffffffu;
     __shared__ __align__(16) NeighWarp sw[NG_WARPS];
     const int lane = threadIdx.x & 31;
@@ -341,6 +342,7 @@ k_neigh(const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ items,
 __global__ void k_neigh_offsets(const int32_t *__restrict__ off32, int64_t n,
                                 int64_t *__restrict__ off64)
 {
+    nb_grid_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n;
          i += (int64_t)gridDim.x * blockDim.x)
         off64[i] = off32[i];
@@ -406,6 +408,7 @@ __device__ __forceinline__ void sort_run(int32_t *a, int32_t len, int lane)
 __global__ void __launch_bounds__(256)
 k_neigh_sort(const int32_t *__restrict__ off, int64_t n, int32_t *__restrict__ idx)
 {
+    nb_grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n;
@@ -449,15 +452,15 @@ static int neigh_pass(nb_ctx *c, bool fill, double h, int32_t *idx, int64_t cap,
     const int32_t *ss = c->nsys > 1 ? c->sys_sorted : nullptr;
     const int32_t *sr = c->nsys > 1 ? c->sys_root : nullptr;
     if (fill)
-        k_neigh<true><<<blocks, NG_T, 0, c->stream>>>(
-            c->wrec, c->items, c->gfirst, c->gcount, c->gbox, c->n_first, c->n_count, c->perm,
-            c->p_hi, c->p_lo, c->p_x64, c->cnt, h, h * h, c->root, c->ccount, c->cstart, idx, cap,
-            c->wq, c->wq_cap, c->n, c->max_items, ss, sr, c->err);
+        nb_launch(k_neigh<true>, blocks, NG_T, 0, nb_queue(c), c->wrec, c->items, c->gfirst,
+                  c->gcount, c->gbox, c->n_first, c->n_count, c->perm, c->p_hi, c->p_lo, c->p_x64,
+                  c->cnt, h, h * h, c->root, c->ccount, c->cstart, idx, cap, c->wq, c->wq_cap,
+                  c->n, c->max_items, ss, sr, c->err);
     else
-        k_neigh<false><<<blocks, NG_T, 0, c->stream>>>(
-            c->wrec, c->items, c->gfirst, c->gcount, c->gbox, c->n_first, c->n_count, c->perm,
-            c->p_hi, c->p_lo, c->p_x64, c->cnt, h, h * h, c->root, c->ccount, nullptr, nullptr, 0,
-            c->wq, c->wq_cap, c->n, c->max_items, ss, sr, c->err);
+        nb_launch(k_neigh<false>, blocks, NG_T, 0, nb_queue(c), c->wrec, c->items, c->gfirst,
+                  c->gcount, c->gbox, c->n_first, c->n_count, c->perm, c->p_hi, c->p_lo, c->p_x64,
+                  c->cnt, h, h * h, c->root, c->ccount, nullptr, nullptr, 0, c->wq, c->wq_cap,
+                  c->n, c->max_items, ss, sr, c->err);
     nb_launched(c, "k_neigh");
     return nb_read_err(c, bits);
 }
@@ -480,8 +483,8 @@ int nb_neigh_run(nb_ctx *c, double h, int n_crit, int64_t *off, int32_t *idx, in
         if (bits) return nb_err_code(bits);
         // offsets in caller order (the count array is in caller order)
         nb_exclusive_scan(c, c->ccount, c->cstart, n + 1, nullptr, &c->cnt[CNT_LIST_TOT]);
-        k_neigh_offsets<<<nb_grid(n + 1, 256, c->num_sms * 8), 256, 0, c->stream>>>(c->cstart, n,
-                                                                                 off);
+        nb_launch(k_neigh_offsets, nb_grid(n + 1, 256, c->num_sms * 8), 256, 0, nb_queue(c),
+                  c->cstart, n, off);
         nb_launched(c, "k_neigh_offsets");
         long long tot = 0;
         CK_RET(cudaMemcpyAsync(&tot, &c->cnt[CNT_LIST_TOT], sizeof(long long),
@@ -493,7 +496,7 @@ int nb_neigh_run(nb_ctx *c, double h, int n_crit, int64_t *off, int32_t *idx, in
         rc = neigh_pass(c, true, h, idx, cap, &bits);
         if (rc) return rc;
         if (bits) return bits & NB_EF_BOUNDS ? NB_ERR_INTERNAL : nb_err_code(bits);
-        k_neigh_sort<<<c->num_sms * 8, 256, 0, c->stream>>>(c->cstart, n, idx);
+        nb_launch(k_neigh_sort, c->num_sms * 8, 256, 0, nb_queue(c), c->cstart, n, idx);
         nb_launched(c, "k_neigh_sort");
         CK_RET(cudaStreamSynchronize(c->stream));
         return cudaGetLastError() == cudaSuccess ? NB_OK : NB_ERR_CUDA;

@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(SCAN_T)
 k_scan_reduce(const int32_t *__restrict__ in, int64_t n_max,
               const long long *__restrict__ n_dev, int32_t *__restrict__ bsum)
 {
+    nb_grid_wait();
     const int64_t n = eff_n(n_max, n_dev);
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     int32_t s = 0;
@@ -87,6 +88,7 @@ k_scan_apply(const int32_t *__restrict__ in, int32_t *__restrict__ out,
              int64_t n_max, const long long *__restrict__ n_dev,
              const int32_t *__restrict__ bsum, long long *__restrict__ total_dev)
 {
+    nb_grid_wait();
     static_assert(SCAN_I == 8, "two 16-byte vectors per thread");
     const int64_t n = eff_n(n_max, n_dev);
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
@@ -143,14 +145,14 @@ void nb_exclusive_scan(nb_ctx *c, const int32_t *in, int32_t *out, int64_t n_max
 {
     const int nb = (int)((n_max + SCAN_TILE - 1) / SCAN_TILE);
     const int g = nb > 0 ? nb : 1;
-    k_scan_reduce<<<g, SCAN_T, 0, c->stream>>>(in, n_max, n_dev, c->scan_bsum);
+    nb_launch(k_scan_reduce, g, SCAN_T, 0, nb_queue(c), in, n_max, n_dev, c->scan_bsum);
     nb_launched(c, "k_scan_reduce");
     if (((uintptr_t)in & 15u) == 0 && ((uintptr_t)out & 15u) == 0)
-        k_scan_apply<true><<<g, SCAN_T, 0, c->stream>>>(in, out, n_max, n_dev, c->scan_bsum,
-                                                        total_dev);
+        nb_launch(k_scan_apply<true>, g, SCAN_T, 0, nb_queue(c), in, out, n_max, n_dev,
+                  c->scan_bsum, total_dev);
     else
-        k_scan_apply<false><<<g, SCAN_T, 0, c->stream>>>(in, out, n_max, n_dev, c->scan_bsum,
-                                                         total_dev);
+        nb_launch(k_scan_apply<false>, g, SCAN_T, 0, nb_queue(c), in, out, n_max, n_dev,
+                  c->scan_bsum, total_dev);
     nb_launched(c, "k_scan_apply");
 }
 
@@ -164,6 +166,7 @@ __global__ void __launch_bounds__(RS_T)
 k_rs_hist(const uint64_t *__restrict__ key, int64_t n, int shift,
           uint32_t *__restrict__ hist, int nb)
 {
+    nb_grid_wait();
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -224,6 +227,7 @@ k_rs_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
              long long *__restrict__ cnt, unsigned *__restrict__ err, uint32_t *status,
              const uint32_t *__restrict__ ghist, uint32_t *tilectr)
 {
+    nb_grid_wait();
     constexpr int TILE = RS_T * I;
     extern __shared__ __align__(16) unsigned char rs_stage[];
     uint64_t *sk = (uint64_t *)rs_stage;
@@ -404,6 +408,7 @@ static void rs_setup()
 __global__ void __launch_bounds__(RS_T)
 k_rs_ghist(const uint64_t *__restrict__ key, int64_t n, uint32_t *__restrict__ ghist)
 {
+    nb_grid_wait();
     __shared__ uint32_t h[8][256];
     for (int i = threadIdx.x; i < 8 * 256; i += RS_T) (&h[0][0])[i] = 0u;
     __syncthreads();
@@ -434,12 +439,12 @@ void nb_radix_sort(nb_ctx *c, int64_t n)
         uint32_t *tctr = ghist + 8 * 256;
         cudaMemsetAsync(c->rs_status, 0, sizeof(uint32_t) * ((int64_t)nb * 256 * 8 + 8 * 256 + 8),
                         c->stream);
-        k_rs_ghist<<<c->num_sms * 4, RS_T, 0, c->stream>>>(ka, n, ghist);
+        nb_launch(k_rs_ghist, c->num_sms * 4, RS_T, 0, nb_queue(c), ka, n, ghist);
         nb_launched(c, "k_rs_ghist");
         for (int pass = 0; pass < 8; pass++) {
-            k_rs_scatter<true, RS_I1><<<nb, RS_T, rs_smem(RS_I1), c->stream>>>(
-                ka, va, kb, vb, nullptr, n, 8 * pass, nb, c->cnt, c->err,
-                c->rs_status + (int64_t)pass * nb * 256, ghist + 256 * pass, tctr + pass);
+            nb_launch(k_rs_scatter<true, RS_I1>, nb, RS_T, rs_smem(RS_I1), nb_queue(c), ka, va, kb,
+                      vb, nullptr, n, 8 * pass, nb, c->cnt, c->err,
+                      c->rs_status + (int64_t)pass * nb * 256, ghist + 256 * pass, tctr + pass);
             nb_launched(c, "k_rs_scatter");
             uint64_t *tk = ka; ka = kb; kb = tk;
             uint32_t *tv = va; va = vb; vb = tv;
@@ -448,13 +453,12 @@ void nb_radix_sort(nb_ctx *c, int64_t n)
     }
     for (int pass = 0; pass < 8; pass++) {
         const int shift = 8 * pass;
-        k_rs_hist<<<nb16, RS_T, 0, c->stream>>>(ka, n, shift, c->sort_hist, nb16);
+        nb_launch(k_rs_hist, nb16, RS_T, 0, nb_queue(c), ka, n, shift, c->sort_hist, nb16);
         nb_launched(c, "k_rs_hist");
         nb_exclusive_scan(c, (const int32_t *)c->sort_hist, (int32_t *)c->sort_hist,
                           (int64_t)256 * nb16, nullptr, nullptr);
-        k_rs_scatter<false><<<nb16, RS_T, RS_SMEM, c->stream>>>(ka, va, kb, vb, c->sort_hist, n,
-                                                                shift, nb16, c->cnt, c->err,
-                                                                nullptr, nullptr, nullptr);
+        nb_launch(k_rs_scatter<false>, nb16, RS_T, RS_SMEM, nb_queue(c), ka, va, kb, vb,
+                  c->sort_hist, n, shift, nb16, c->cnt, c->err, nullptr, nullptr, nullptr);
         nb_launched(c, "k_rs_scatter");
         uint64_t *tk = ka; ka = kb; kb = tk;
         uint32_t *tv = va; va = vb; vb = tv;
@@ -469,11 +473,13 @@ void nb_exclusive_scan_raw(const int32_t *in, int32_t *out, int64_t n_max, int32
 {
     const int nb = (int)((n_max + SCAN_TILE - 1) / SCAN_TILE);
     const int g = nb > 0 ? nb : 1;
-    k_scan_reduce<<<g, SCAN_T, 0, s>>>(in, n_max, nullptr, bsum);
+    nb_launch(k_scan_reduce, g, SCAN_T, 0, nb_queue(s, n_max), in, n_max, nullptr, bsum);
     if (((uintptr_t)in & 15u) == 0 && ((uintptr_t)out & 15u) == 0)
-        k_scan_apply<true><<<g, SCAN_T, 0, s>>>(in, out, n_max, nullptr, bsum, nullptr);
+        nb_launch(k_scan_apply<true>, g, SCAN_T, 0, nb_queue(s, n_max), in, out, n_max, nullptr,
+                  bsum, nullptr);
     else
-        k_scan_apply<false><<<g, SCAN_T, 0, s>>>(in, out, n_max, nullptr, bsum, nullptr);
+        nb_launch(k_scan_apply<false>, g, SCAN_T, 0, nb_queue(s, n_max), in, out, n_max, nullptr,
+                  bsum, nullptr);
 }
 
 // keys/idx hold the input and, after the 8 passes, the sorted output;
@@ -496,10 +502,10 @@ void nb_radix_sort_passes(uint64_t *keys, uint64_t *keys_alt, uint32_t *idx, uin
     uint32_t *va = idx, *vb = idx_alt;
     for (int pass = 0; pass < passes; pass++) {
         const int shift = 8 * pass;
-        k_rs_hist<<<nb, RS_T, 0, s>>>(ka, n, shift, hist, nb);
+        nb_launch(k_rs_hist, nb, RS_T, 0, nb_queue(s, n), ka, n, shift, hist, nb);
         nb_exclusive_scan_raw((const int32_t *)hist, (int32_t *)hist, (int64_t)256 * nb, bsum, s);
-        k_rs_scatter<false><<<nb, RS_T, RS_SMEM, s>>>(ka, va, kb, vb, hist, n, shift, nb, nullptr,
-                                                      nullptr, nullptr, nullptr, nullptr);
+        nb_launch(k_rs_scatter<false>, nb, RS_T, RS_SMEM, nb_queue(s, n), ka, va, kb, vb, hist, n,
+                  shift, nb, nullptr, nullptr, nullptr, nullptr, nullptr);
         uint64_t *tk = ka; ka = kb; kb = tk;
         uint32_t *tv = va; va = vb; vb = tv;
     }

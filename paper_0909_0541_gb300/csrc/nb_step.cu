@@ -27,6 +27,7 @@ template <bool V4>
 __global__ void __launch_bounds__(256)
 k_kick(double *__restrict__ vel, const float *__restrict__ acc, int64_t m, double h)
 {
+    nb_grid_wait();
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t nt = (int64_t)gridDim.x * blockDim.x;
     int64_t tail = 0;
@@ -51,6 +52,7 @@ template <bool V4>
 __global__ void __launch_bounds__(256)
 k_drift(double *__restrict__ pos, const double *__restrict__ vel, int64_t m, double dt)
 {
+    nb_grid_wait();
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t nt = (int64_t)gridDim.x * blockDim.x;
     int64_t tail = 0;
@@ -81,6 +83,7 @@ __global__ void __launch_bounds__(256)
 k_kick_kick_drift(double *__restrict__ pos, double *__restrict__ vel,
                   const float *__restrict__ acc, int64_t m, double h, double dt)
 {
+    nb_grid_wait();
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t nt = (int64_t)gridDim.x * blockDim.x;
     int64_t tail = 0;
@@ -119,9 +122,9 @@ void nb_launch_kick(nb_ctx *c, double *vel, const float *acc, int64_t n, double 
     const bool v4 = aligned16(vel) && aligned16(acc);
     const int grid = nb_grid(v4 ? (3 * n + 3) / 4 : 3 * n, 256, c->num_sms * 8);
     if (v4)
-        k_kick<true><<<grid, 256, 0, c->stream>>>(vel, acc, 3 * n, h);
+        nb_launch(k_kick<true>, grid, 256, 0, nb_queue(c), vel, acc, 3 * n, h);
     else
-        k_kick<false><<<grid, 256, 0, c->stream>>>(vel, acc, 3 * n, h);
+        nb_launch(k_kick<false>, grid, 256, 0, nb_queue(c), vel, acc, 3 * n, h);
     nb_launched(c, "k_kick");
 }
 
@@ -130,9 +133,9 @@ void nb_launch_drift(nb_ctx *c, double *pos, const double *vel, int64_t n, doubl
     const bool v4 = aligned16(pos) && aligned16(vel);
     const int grid = nb_grid(v4 ? (3 * n + 3) / 4 : 3 * n, 256, c->num_sms * 8);
     if (v4)
-        k_drift<true><<<grid, 256, 0, c->stream>>>(pos, vel, 3 * n, dt);
+        nb_launch(k_drift<true>, grid, 256, 0, nb_queue(c), pos, vel, 3 * n, dt);
     else
-        k_drift<false><<<grid, 256, 0, c->stream>>>(pos, vel, 3 * n, dt);
+        nb_launch(k_drift<false>, grid, 256, 0, nb_queue(c), pos, vel, 3 * n, dt);
     nb_launched(c, "k_drift");
 }
 
@@ -142,8 +145,9 @@ void nb_launch_kick_kick_drift(nb_ctx *c, double *pos, double *vel, const float 
     const bool v4 = aligned16(pos) && aligned16(vel) && aligned16(acc);
     const int grid = nb_grid(v4 ? (3 * n + 3) / 4 : 3 * n, 256, c->num_sms * 8);
     if (v4)
-        k_kick_kick_drift<true><<<grid, 256, 0, c->stream>>>(pos, vel, acc, 3 * n, h, dt);
+        nb_launch(k_kick_kick_drift<true>, grid, 256, 0, nb_queue(c), pos, vel, acc, 3 * n, h, dt);
     else
-        k_kick_kick_drift<false><<<grid, 256, 0, c->stream>>>(pos, vel, acc, 3 * n, h, dt);
+        nb_launch(k_kick_kick_drift<false>, grid, 256, 0, nb_queue(c), pos, vel, acc, 3 * n, h,
+                  dt);
     nb_launched(c, "k_kick_kick_drift");
 }

@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(256)
 k_bbox(const double *__restrict__ pos, int64_t n, double *__restrict__ part,
        unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     bbox_block(pos, n, part, err);
 }
 
@@ -123,6 +124,7 @@ __device__ __forceinline__ void root_block(const double *part, int nblk, double 
 __global__ void __launch_bounds__(256)
 k_root(const double *__restrict__ part, int nblk, double *__restrict__ root)
 {
+    nb_grid_wait();
     root_block(part, nblk, root);
 }
 
@@ -134,6 +136,7 @@ __global__ void __launch_bounds__(256)
 k_bbox_root(const double *__restrict__ pos, int64_t n, double *part, unsigned *__restrict__ err,
             long long *__restrict__ cnt, double *__restrict__ root)
 {
+    nb_grid_wait();
     __shared__ bool last;
     bbox_block(pos, n, part, err);
     __threadfence();   // this block's partial before its arrival
@@ -256,6 +259,7 @@ k_keys(const double *__restrict__ pos, int64_t n, const double *__restrict__ roo
        const int32_t *__restrict__ sys_of, uint64_t *__restrict__ key, uint32_t *__restrict__ idx,
        int hilbert)
 {
+    nb_grid_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double *root = roots + (sys_of ? 8 * (int64_t)sys_of[i] : 0);
@@ -276,6 +280,7 @@ k_gather(const double *__restrict__ pos, const float *__restrict__ mass, int64_t
          double *__restrict__ x64, float4 *__restrict__ p_hi, float4 *__restrict__ p_lo,
          long long *__restrict__ cnt, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     const uint32_t i = idx[s];
@@ -306,6 +311,7 @@ __global__ void __launch_bounds__(256)
 k_levels(const uint64_t *__restrict__ key, int64_t n, const int32_t *__restrict__ sys,
          int8_t *__restrict__ clev, int32_t *__restrict__ ccount)
 {
+    nb_grid_wait();
     const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (a >= n) return;
     const int ca = a + 1 < n && (!sys || sys[a] == sys[a + 1]) ? common_levels(key[a], key[a + 1]) : -1;
@@ -363,6 +369,7 @@ k_cells(const uint64_t *__restrict__ key, int64_t n, const int8_t *__restrict__ 
         long long *__restrict__ cnt, const int32_t *__restrict__ sys,
         const int64_t *__restrict__ sys_off, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int deepest = -1;
     if (a < n) deepest = cell_records(a, n, clev, cstart, node_c, n_level, n_first, n_count,
@@ -385,6 +392,7 @@ k_cell_ends(const uint64_t *__restrict__ key, int64_t n, const int32_t *__restri
             long long *__restrict__ cnt, const int32_t *__restrict__ sys,
             const int64_t *__restrict__ sys_off, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int32_t total = (int32_t)cnt[CNT_NODES];
     for (int32_t id = blockIdx.x * blockDim.x + threadIdx.x; id < total;
          id += gridDim.x * blockDim.x) {
@@ -418,6 +426,7 @@ k_parents(const int4 *__restrict__ node_c, long long *__restrict__ cnt,
           int32_t *__restrict__ n_parent, int32_t *__restrict__ n_nchild,
           int32_t *__restrict__ arrive, int32_t *__restrict__ lcount, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int32_t total = (int32_t)cnt[CNT_NODES];
     for (int32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < total;
          u += gridDim.x * blockDim.x) {
@@ -449,6 +458,7 @@ __global__ void __launch_bounds__(DS_T)
 k_depth_hist(const int8_t *__restrict__ depth, const long long *__restrict__ cnt,
              uint32_t *__restrict__ hist, int ntiles)
 {
+    nb_grid_wait();
     __shared__ uint32_t h[32];
     if (threadIdx.x < 32) h[threadIdx.x] = 0;
     __syncthreads();
@@ -471,6 +481,7 @@ k_depth_scatter(const int8_t *__restrict__ depth, long long *__restrict__ cnt,
                 const uint32_t *__restrict__ offs, int ntiles, int32_t *__restrict__ bfs2pid,
                 int32_t *__restrict__ pid2bfs, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     __shared__ uint32_t whist[DS_T / NB_WARP][32];
     __shared__ uint32_t boff[32];
     __shared__ uint32_t lstart[32];
@@ -549,6 +560,7 @@ k_depth_scatter(const int8_t *__restrict__ depth, long long *__restrict__ cnt,
 __global__ void k_level_start(const uint32_t *__restrict__ hist, int ntiles,
                               int32_t *__restrict__ level_start)
 {
+    nb_grid_wait();
     const int d = threadIdx.x;
     if (d <= NB_DEPTHS) level_start[d] = (int32_t)hist[(int64_t)d * ntiles];
 }
@@ -576,6 +588,7 @@ k_bfs_records(const int32_t *__restrict__ bfs2pid, const int32_t *__restrict__ p
               int32_t *__restrict__ cbkt_cnt, int64_t n, int hilbert, double *__restrict__ b_q,
               unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     __shared__ int32_t hb[NB_CBKT];   // cells per moments bucket in this block
     for (int k = threadIdx.x; k < NB_CBKT; k += blockDim.x) hb[k] = 0;
     __syncthreads();
@@ -690,6 +703,7 @@ k_cell_list(const int16_t *__restrict__ cbkt, int32_t *__restrict__ cbkt_cnt,
             long long *__restrict__ cnt, int32_t *__restrict__ clist, int64_t clist_len,
             unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     static_assert(NB_CBKT <= 256, "one bucket per thread");
     __shared__ int32_t start[NB_CBKT + 1];
     __shared__ int32_t local[NB_CBKT];
@@ -857,6 +871,7 @@ k_moments(const int32_t *__restrict__ clist, int64_t clist_len, nb_wrec *__restr
           double *b_mx, double *b_com, double *b_q, int32_t *arrive,
           long long *__restrict__ cnt, unsigned *err)
 {
+    nb_grid_wait();
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int32_t total = (int32_t)cnt[CNT_NODES];
@@ -931,10 +946,11 @@ void nb_launch_build(nb_ctx *c, const double *pos, const float *mass, int64_t n)
 {
     cudaStream_t s = c->stream;
     cudaMemsetAsync(c->cnt, 0, sizeof(long long) * CNT_PP_CUM, s);
-    k_bbox_root<<<c->bbox_blocks, 256, 0, s>>>(pos, n, c->bbox_part, c->err, c->cnt, c->root);
+    nb_launch(k_bbox_root, c->bbox_blocks, 256, 0, nb_queue(c), pos, n, c->bbox_part, c->err,
+              c->cnt, c->root);
     nb_launched(c, "k_bbox_root");
-    k_keys<<<nb_grid(n, 256), 256, 0, s>>>(pos, n, c->root, nullptr, c->keys, c->idx,
-                                           c->key_order);
+    nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(c), pos, n, c->root, nullptr, c->keys,
+              c->idx, c->key_order);
     nb_launched(c, "k_keys");
     nb_radix_sort(c, n);
     build_tail(c, pos, mass, n, nullptr);
@@ -946,6 +962,7 @@ __global__ void __launch_bounds__(256)
 k_sys_of(const int64_t *__restrict__ off, int64_t nsys, int64_t n, int32_t *__restrict__ sys_of,
          unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     for (int64_t sy = blockIdx.x; sy < nsys; sy += gridDim.x) {
         const int64_t a = off[sy], b = off[sy + 1];
         if (threadIdx.x == 0 && (!(b > a) || a < 0 || b > n || (sy == 0 && a != 0) ||
@@ -965,6 +982,7 @@ __global__ void __launch_bounds__(RS_SYS_T)
 k_roots_sys(const double *__restrict__ pos, const int64_t *__restrict__ off, int64_t nsys,
             int64_t n, double *__restrict__ roots, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const long long FLIP = 0x7fffffffffffffffll;
     __shared__ long long s[RS_SYS_T / 32][6];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1030,6 +1048,7 @@ __global__ void __launch_bounds__(256)
 k_sys_key(const uint32_t *__restrict__ idx, const int32_t *__restrict__ sys_of, int64_t n,
           uint64_t *__restrict__ skey, uint32_t *__restrict__ sval)
 {
+    nb_grid_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     skey[i] = (uint64_t)sys_of[idx[i]];
@@ -1043,6 +1062,7 @@ k_sys_apply(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
             uint64_t *__restrict__ key_out, uint32_t *__restrict__ idx_out,
             int32_t *__restrict__ sys_sorted)
 {
+    nb_grid_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const uint32_t j = sval[i];
@@ -1057,6 +1077,7 @@ k_sys_roots(const int32_t *__restrict__ level_start, const int32_t *__restrict__
             const int32_t *__restrict__ n_first, const int32_t *__restrict__ sys_sorted,
             int32_t *__restrict__ sys_root)
 {
+    nb_grid_wait();
     const int32_t nr = level_start[1];
     for (int32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < nr; b += gridDim.x * blockDim.x)
         sys_root[sys_sorted[n_first[bfs2pid[b]]]] = b;
@@ -1068,29 +1089,29 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
     cudaStream_t s = c->stream;
     cudaMemsetAsync(c->cnt, 0, sizeof(long long) * CNT_PP_CUM, s);
     const int gs = (int)(nsys < 65535 ? nsys : 65535);
-    k_sys_of<<<gs, 256, 0, s>>>(off, nsys, n, c->sys_of, c->err);
+    nb_launch(k_sys_of, gs, 256, 0, nb_queue(c), off, nsys, n, c->sys_of, c->err);
     nb_launched(c, "k_sys_of");
-    k_roots_sys<<<gs, RS_SYS_T, 0, s>>>(pos, off, nsys, n, c->root, c->err);
+    nb_launch(k_roots_sys, gs, RS_SYS_T, 0, nb_queue(c), pos, off, nsys, n, c->root, c->err);
     nb_launched(c, "k_roots_sys");
-    k_keys<<<nb_grid(n, 256), 256, 0, s>>>(pos, n, c->root, c->sys_of, c->keys, c->idx,
-                                           c->key_order);
+    nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(c), pos, n, c->root, c->sys_of, c->keys,
+              c->idx, c->key_order);
     nb_launched(c, "k_keys");
     nb_radix_sort(c, n);
     // stable by system on top of the Morton order: (system, key) order
-    k_sys_key<<<nb_grid(n, 256), 256, 0, s>>>(c->idx, c->sys_of, n, c->skey, c->sval);
+    nb_launch(k_sys_key, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, c->sys_of, n, c->skey,
+              c->sval);
     nb_launched(c, "k_sys_key");
     nb_radix_sort_passes(c->skey, c->skey_alt, c->sval, c->sval_alt, c->sort_hist, c->scan_bsum,
                          n, 2, s);
     c->launches += 2 * 5;
-    k_sys_apply<<<nb_grid(n, 256), 256, 0, s>>>(c->keys, c->idx, c->skey, c->sval, n,
-                                                c->keys_alt, c->idx_alt, c->sys_sorted);
+    nb_launch(k_sys_apply, nb_grid(n, 256), 256, 0, nb_queue(c), c->keys, c->idx, c->skey, c->sval,
+              n, c->keys_alt, c->idx_alt, c->sys_sorted);
     nb_launched(c, "k_sys_apply");
     uint64_t *tk = c->keys; c->keys = c->keys_alt; c->keys_alt = tk;
     uint32_t *ti = c->idx; c->idx = c->idx_alt; c->idx_alt = ti;
     build_tail(c, pos, mass, n, c->sys_sorted);
-    k_sys_roots<<<nb_grid(nsys, 256, c->num_sms * 4), 256, 0, s>>>(c->level_start, c->bfs2pid,
-                                                                    c->n_first, c->sys_sorted,
-                                                                    c->sys_root);
+    nb_launch(k_sys_roots, nb_grid(nsys, 256, c->num_sms * 4), 256, 0, nb_queue(c), c->level_start,
+              c->bfs2pid, c->n_first, c->sys_sorted, c->sys_root);
     nb_launched(c, "k_sys_roots");
 }
 
@@ -1098,47 +1119,46 @@ static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t 
                        const int32_t *sys_sorted)
 {
     cudaStream_t s = c->stream;
-    k_gather<<<nb_grid(n, 256), 256, 0, s>>>(pos, mass, n, c->idx, c->perm, c->p_x64,
-                                             c->p_hi, c->p_lo, c->cnt, c->err);
+    nb_launch(k_gather, nb_grid(n, 256), 256, 0, nb_queue(c), pos, mass, n, c->idx, c->perm,
+              c->p_x64, c->p_hi, c->p_lo, c->cnt, c->err);
     nb_launched(c, "k_gather");
-    k_levels<<<nb_grid(n, 256), 256, 0, s>>>(c->keys, n, sys_sorted, c->clev, c->ccount);
+    nb_launch(k_levels, nb_grid(n, 256), 256, 0, nb_queue(c), c->keys, n, sys_sorted, c->clev,
+              c->ccount);
     nb_launched(c, "k_levels");
     nb_exclusive_scan(c, c->ccount, c->cstart, n, nullptr, &c->cnt[CNT_CELLS]);
-    k_cells<<<nb_grid(n, 256), 256, 0, s>>>(c->keys, n, c->clev, c->cstart, c->node_c,
-                                            c->n_level, c->n_first, c->n_count, c->n_parent,
-                                            c->n_nchild, c->n_depth, c->cnt, sys_sorted,
-                                            c->sys_off, c->err);
+    nb_launch(k_cells, nb_grid(n, 256), 256, 0, nb_queue(c), c->keys, n, c->clev, c->cstart,
+              c->node_c, c->n_level, c->n_first, c->n_count, c->n_parent, c->n_nchild, c->n_depth,
+              c->cnt, sys_sorted, c->sys_off, c->err);
     nb_launched(c, "k_cells");
     const int gcap = c->num_sms * 16;
-    k_cell_ends<<<nb_grid(c->max_nodes, 256, gcap), 256, 0, s>>>(
-        c->keys, n, c->cstart, c->n_level, c->n_first, c->node_c, c->n_count, c->cnt, sys_sorted,
-        c->sys_off, c->err);
+    nb_launch(k_cell_ends, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->keys, n,
+              c->cstart, c->n_level, c->n_first, c->node_c, c->n_count, c->cnt, sys_sorted,
+              c->sys_off, c->err);
     nb_launched(c, "k_cell_ends");
-    k_parents<<<nb_grid(c->max_nodes, 256, gcap), 256, 0, s>>>(c->node_c, c->cnt, c->n_parent,
-                                                               c->n_nchild, c->arrive, c->lcount,
-                                                               c->err);
+    nb_launch(k_parents, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->node_c, c->cnt,
+              c->n_parent, c->n_nchild, c->arrive, c->lcount, c->err);
     nb_launched(c, "k_parents");
     // level order
     const int nt = (int)c->dtiles;
-    k_depth_hist<<<nt, DS_T, 0, s>>>(c->n_depth, c->cnt, c->dhist, nt);
+    nb_launch(k_depth_hist, nt, DS_T, 0, nb_queue(c), c->n_depth, c->cnt, c->dhist, nt);
     nb_launched(c, "k_depth_hist");
     nb_exclusive_scan(c, (const int32_t *)c->dhist, (int32_t *)c->dhist,
                       (int64_t)NB_DEPTHS * nt, nullptr, nullptr);
-    k_depth_scatter<<<nt, DS_T, 0, s>>>(c->n_depth, c->cnt, c->dhist, nt, c->bfs2pid, c->pid2bfs,
-                                        c->err);
+    nb_launch(k_depth_scatter, nt, DS_T, 0, nb_queue(c), c->n_depth, c->cnt, c->dhist, nt,
+              c->bfs2pid, c->pid2bfs, c->err);
     nb_launched(c, "k_depth_scatter");
-    k_level_start<<<1, 32, 0, s>>>(c->dhist, nt, c->level_start);
+    nb_launch(k_level_start, 1, 32, 0, nb_queue(c), c->dhist, nt, c->level_start);
     nb_launched(c, "k_level_start");
     cudaMemsetAsync(c->cbkt_cnt, 0, sizeof(int32_t) * 2 * NB_CBKT, s);
-    k_bfs_records<<<nb_grid(c->max_nodes, 256, gcap), 256, 0, s>>>(
-        c->bfs2pid, c->pid2bfs, c->node_c, c->n_first, c->n_nchild, c->n_parent, c->n_depth,
-        c->keys, c->root, sys_sorted, c->p_hi, c->p_lo, c->p_x64, c->cnt, c->wrec, c->b_mass,
-        c->b_mx, c->b_com, c->b_up, c->lcount, c->cbkt, c->cbkt_cnt, n, c->key_order,
-        c->quad ? c->b_q : nullptr, c->err);
+    nb_launch(k_bfs_records, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->bfs2pid,
+              c->pid2bfs, c->node_c, c->n_first, c->n_nchild, c->n_parent, c->n_depth, c->keys,
+              c->root, sys_sorted, c->p_hi, c->p_lo, c->p_x64, c->cnt, c->wrec, c->b_mass, c->b_mx,
+              c->b_com, c->b_up, c->lcount, c->cbkt, c->cbkt_cnt, n, c->key_order,
+              c->quad ? c->b_q : nullptr, c->err);
     nb_launched(c, "k_bfs_records");
     const int cl_blocks = (int)((c->max_nodes + CL_TILE - 1) / CL_TILE);
-    k_cell_list<<<cl_blocks > 0 ? cl_blocks : 1, 256, 0, s>>>(c->cbkt, c->cbkt_cnt, c->cnt,
-                                                               c->clist, c->clist_len, c->err);
+    nb_launch(k_cell_list, cl_blocks > 0 ? cl_blocks : 1, 256, 0, nb_queue(c), c->cbkt,
+              c->cbkt_cnt, c->cnt, c->clist, c->clist_len, c->err);
     nb_launched(c, "k_cell_list");
     static int mblocks = 0, qblocks = 0;
     if (mblocks == 0) {
@@ -1148,13 +1168,13 @@ static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t 
         if (qblocks < 1) qblocks = 1;
     }
     if (c->quad && c->b_q)
-        k_moments<true><<<c->num_sms * qblocks, 256, 0, s>>>(
-            c->clist, c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass, c->b_mx, c->b_com,
-            c->b_q, c->arrive, c->cnt, c->err);
+        nb_launch(k_moments<true>, c->num_sms * qblocks, 256, 0, nb_queue(c), c->clist,
+                  c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass, c->b_mx, c->b_com, c->b_q,
+                  c->arrive, c->cnt, c->err);
     else
-        k_moments<false><<<c->num_sms * mblocks, 256, 0, s>>>(
-            c->clist, c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass, c->b_mx, c->b_com,
-            nullptr, c->arrive, c->cnt, c->err);
+        nb_launch(k_moments<false>, c->num_sms * mblocks, 256, 0, nb_queue(c), c->clist,
+                  c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass, c->b_mx, c->b_com, nullptr,
+                  c->arrive, c->cnt, c->err);
     nb_launched(c, "k_moments");
 }
 
@@ -1164,6 +1184,7 @@ k_group_flags(const int32_t *__restrict__ n_count, const int32_t *__restrict__ n
               long long *__restrict__ cnt, int n_crit, int32_t *__restrict__ flag,
               unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int32_t total = (int32_t)cnt[CNT_NODES];
     for (int32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < total;
          u += gridDim.x * blockDim.x) {
@@ -1179,6 +1200,7 @@ k_group_scatter(const int32_t *__restrict__ gid, const int32_t *__restrict__ n_f
                 int32_t *__restrict__ gnode, int32_t *__restrict__ gfirst,
                 int32_t *__restrict__ gcount, int64_t n, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int32_t total = (int32_t)cnt[CNT_NODES];
     for (int32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < total;
          u += gridDim.x * blockDim.x) {
@@ -1218,6 +1240,7 @@ k_group_boxes(const int32_t *__restrict__ gfirst, const int32_t *__restrict__ gc
               float theta, const float *__restrict__ theta_g, float4 *__restrict__ gbox,
               int32_t *__restrict__ item_cnt, int iblock, int64_t n, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int32_t G = (int32_t)cnt[CNT_GROUPS];
@@ -1281,6 +1304,7 @@ k_items(const int32_t *__restrict__ item_off, const int32_t *__restrict__ gcount
         long long *__restrict__ cnt, int32_t *__restrict__ items, int iblock, int64_t max_items,
         unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int32_t G = (int32_t)cnt[CNT_GROUPS];
     for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G;
          g += gridDim.x * blockDim.x) {
@@ -1315,6 +1339,7 @@ __global__ void __launch_bounds__(256)
 k_group_theta(const float *__restrict__ theta_g, const long long *__restrict__ cnt,
               float4 *__restrict__ gbox)
 {
+    nb_grid_wait();
     const int32_t G = (int32_t)cnt[CNT_GROUPS];
     for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x)
         gbox[3 * (int64_t)g + 2].w = __double2float_rn(__ddiv_rn(1.0, (double)theta_g[g]));
@@ -1322,32 +1347,29 @@ k_group_theta(const float *__restrict__ theta_g, const long long *__restrict__ c
 
 void nb_launch_group_theta(nb_ctx *c, const float *theta_g)
 {
-    k_group_theta<<<nb_grid(c->max_n, 256, c->num_sms * 8), 256, 0, c->stream>>>(theta_g, c->cnt,
-                                                                                c->gbox);
+    nb_launch(k_group_theta, nb_grid(c->max_n, 256, c->num_sms * 8), 256, 0, nb_queue(c), theta_g,
+              c->cnt, c->gbox);
     nb_launched(c, "k_group_theta");
 }
 
 void nb_launch_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g)
 {
-    cudaStream_t s = c->stream;
     const int gcap = c->num_sms * 16;
-    k_group_flags<<<nb_grid(c->max_nodes, 256, gcap), 256, 0, s>>>(
-        c->n_count, c->n_parent, c->cnt, n_crit, c->gflag, c->err);
+    nb_launch(k_group_flags, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->n_count,
+              c->n_parent, c->cnt, n_crit, c->gflag, c->err);
     nb_launched(c, "k_group_flags");
     nb_exclusive_scan(c, c->gflag, c->gflag, c->max_nodes, &c->cnt[CNT_NODES],
                       &c->cnt[CNT_GROUPS]);
-    k_group_scatter<<<nb_grid(c->max_nodes, 256, gcap), 256, 0, s>>>(
-        c->gflag, c->n_first, c->n_count, c->cnt, c->gnode, c->gfirst, c->gcount, c->n, c->err);
+    nb_launch(k_group_scatter, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->gflag,
+              c->n_first, c->n_count, c->cnt, c->gnode, c->gfirst, c->gcount, c->n, c->err);
     nb_launched(c, "k_group_scatter");
-    k_group_boxes<<<c->num_sms * 16, 256, 0, s>>>(
-        c->gfirst, c->gcount, c->p_hi, c->cnt, theta, theta_g, c->gbox, c->item_cnt,
-        c->item_rows * NB_WARP, c->n, c->err);
+    nb_launch(k_group_boxes, c->num_sms * 16, 256, 0, nb_queue(c), c->gfirst, c->gcount, c->p_hi,
+              c->cnt, theta, theta_g, c->gbox, c->item_cnt, c->item_rows * NB_WARP, c->n, c->err);
     nb_launched(c, "k_group_boxes");
     nb_exclusive_scan(c, c->item_cnt, c->item_cnt, c->max_n, &c->cnt[CNT_GROUPS],
                       &c->cnt[CNT_ITEMS]);
-    k_items<<<nb_grid(c->max_n, 256, gcap), 256, 0, s>>>(c->item_cnt, c->gcount, c->cnt,
-                                                          c->items, c->item_rows * NB_WARP,
-                                                          c->max_items, c->err);
+    nb_launch(k_items, nb_grid(c->max_n, 256, gcap), 256, 0, nb_queue(c), c->item_cnt, c->gcount,
+              c->cnt, c->items, c->item_rows * NB_WARP, c->max_items, c->err);
     nb_launched(c, "k_items");
 }
 
@@ -1356,8 +1378,9 @@ void nb_launch_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g)
 void nb_launch_keys_raw(const double *pos, int64_t n, double *part, int nblk, double *root,
                         uint64_t *keys, uint32_t *idx, unsigned *err, cudaStream_t s)
 {
-    k_bbox<<<nblk, 256, 0, s>>>(pos, n, part, err);
-    k_root<<<1, 256, 0, s>>>(part, nblk, root);
-    k_keys<<<nb_grid(n, 256), 256, 0, s>>>(pos, n, root, nullptr, keys, idx, 0);
+    nb_launch(k_bbox, nblk, 256, 0, nb_queue(s, n), pos, n, part, err);
+    nb_launch(k_root, 1, 256, 0, nb_queue(s, n), part, nblk, root);
+    nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(s, n), pos, n, root, nullptr, keys, idx,
+              0);
 }
 

@@ -40,6 +40,7 @@ k_walk(const nb_wrec *__restrict__ wrec,
        const int32_t *__restrict__ gfirst, const int32_t *__restrict__ sys_sorted,
        const int32_t *__restrict__ sys_root)
 {
+    nb_grid_wait();
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -86,6 +87,7 @@ k_group_features_tree(const int32_t *__restrict__ gnode, const int32_t *__restri
                       const int32_t *__restrict__ sys_sorted, long long *__restrict__ cnt,
                       float *__restrict__ feat, int64_t n, unsigned *__restrict__ err)
 {
+    nb_grid_wait();
     const int32_t G = (int32_t)cnt[CNT_GROUPS];
     const int32_t total = (int32_t)cnt[CNT_NODES];
     for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
@@ -118,9 +120,9 @@ k_group_features_tree(const int32_t *__restrict__ gnode, const int32_t *__restri
 
 void nb_launch_features_tree(nb_ctx *c, float *feat)
 {
-    k_group_features_tree<<<nb_grid(c->max_n, 256, c->num_sms * 8), 256, 0, c->stream>>>(
-        c->gnode, c->gfirst, c->gcount, c->gbox, c->root, c->n_depth,
-        c->nsys > 1 ? c->sys_sorted : nullptr, c->cnt, feat, c->n, c->err);
+    nb_launch(k_group_features_tree, nb_grid(c->max_n, 256, c->num_sms * 8), 256, 0, nb_queue(c),
+              c->gnode, c->gfirst, c->gcount, c->gbox, c->root, c->n_depth,
+              c->nsys > 1 ? c->sys_sorted : nullptr, c->cnt, feat, c->n, c->err);
     nb_launched(c, "k_group_features_tree");
 }
 
@@ -152,17 +154,17 @@ void nb_launch_walk(nb_ctx *c)
     cudaMemsetAsync(&c->cnt[CNT_QMAX], 0, sizeof(long long), c->stream);
     const int blocks = c->walk_warps / WALK_WARPS;
     if (c->quad && c->b_q && c->list_q)
-        k_walk<false, true><<<blocks, WALK_T, 0, c->stream>>>(
-            c->wrec, c->pid2bfs, c->gnode, c->gcount, c->gbox, c->cnt, c->glen, c->gcells,
-            c->list_id, c->list_xm, c->b_q, c->list_q, c->list_cap, c->list_alloc, c->wq,
-            c->wq_cap, c->err, nullptr, c->root, c->n_depth, c->gfirst,
-            c->nsys > 1 ? c->sys_sorted : nullptr, c->nsys > 1 ? c->sys_root : nullptr);
+        nb_launch(k_walk<false, true>, blocks, WALK_T, 0, nb_queue(c), c->wrec, c->pid2bfs,
+                  c->gnode, c->gcount, c->gbox, c->cnt, c->glen, c->gcells, c->list_id, c->list_xm,
+                  c->b_q, c->list_q, c->list_cap, c->list_alloc, c->wq, c->wq_cap, c->err, nullptr,
+                  c->root, c->n_depth, c->gfirst, c->nsys > 1 ? c->sys_sorted : nullptr,
+                  c->nsys > 1 ? c->sys_root : nullptr);
     else
-        k_walk<false><<<blocks, WALK_T, 0, c->stream>>>(
-            c->wrec, c->pid2bfs, c->gnode, c->gcount, c->gbox, c->cnt, c->glen, c->gcells,
-            c->list_id, c->list_xm, nullptr, nullptr, c->list_cap, c->list_alloc, c->wq,
-            c->wq_cap, c->err, nullptr, c->root, c->n_depth, c->gfirst,
-            c->nsys > 1 ? c->sys_sorted : nullptr, c->nsys > 1 ? c->sys_root : nullptr);
+        nb_launch(k_walk<false>, blocks, WALK_T, 0, nb_queue(c), c->wrec, c->pid2bfs, c->gnode,
+                  c->gcount, c->gbox, c->cnt, c->glen, c->gcells, c->list_id, c->list_xm, nullptr,
+                  nullptr, c->list_cap, c->list_alloc, c->wq, c->wq_cap, c->err, nullptr, c->root,
+                  c->n_depth, c->gfirst, c->nsys > 1 ? c->sys_sorted : nullptr,
+                  c->nsys > 1 ? c->sys_root : nullptr);
     nb_launched(c, "k_walk");
 }
 
@@ -172,11 +174,9 @@ void nb_launch_probe(nb_ctx *c, float *feat)
 {
     cudaMemsetAsync(&c->cnt[CNT_WALK_Q], 0, sizeof(long long), c->stream);
     const int blocks = c->walk_warps / WALK_WARPS;
-    k_walk<true><<<blocks, WALK_T, 0, c->stream>>>(
-        c->wrec, c->pid2bfs, c->gnode, c->gcount, c->gbox, c->cnt,
-        c->glen, c->gcells, nullptr, nullptr, nullptr, nullptr, 0, 0, c->wq, c->wq_cap, c->err,
-        feat, c->root,
-        c->n_depth, c->gfirst, c->nsys > 1 ? c->sys_sorted : nullptr,
-        c->nsys > 1 ? c->sys_root : nullptr);
+    nb_launch(k_walk<true>, blocks, WALK_T, 0, nb_queue(c), c->wrec, c->pid2bfs, c->gnode,
+              c->gcount, c->gbox, c->cnt, c->glen, c->gcells, nullptr, nullptr, nullptr, nullptr,
+              0, 0, c->wq, c->wq_cap, c->err, feat, c->root, c->n_depth, c->gfirst,
+              c->nsys > 1 ? c->sys_sorted : nullptr, c->nsys > 1 ? c->sys_root : nullptr);
     nb_launched(c, "k_walk");
 }
