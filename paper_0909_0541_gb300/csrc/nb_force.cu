@@ -1,7 +1,8 @@
 // nb_force.cu -- Eq. (gravity) summed over each group's interaction list.
 //
 // Work items cut a group's members into 64-target items (two targets per
-// lane) while 64 or more remain, then one 32-target item if more than 32
+// lane; 32, 16 or 8 targets with few particles, see nb_item_block) while 64
+// or more remain, then one 32-target item if more than 32
 // remain, then a tail of at most 32 targets rounded up to a power of two m'.
 // An item of m' <= 32 targets runs as S source streams: the warp is S rows
 // of W = 32/S lanes, stream s takes entries s*W .. s*W+W-1 of every

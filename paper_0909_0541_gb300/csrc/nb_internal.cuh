@@ -189,7 +189,7 @@ struct nb_ctx {
     int32_t *gnode, *gfirst, *gcount, *glen, *gcells;
     float4 *gbox;     // 3 per group
     int32_t *items;   // force work items: (group, first member | one-warp-row flag)
-    int item_rows;    // targets per item: 32 x item_rows (1 or 2)
+    int item_rows;    // targets per item: at most 32 x item_rows (nb_item_block)
     int force_tile;   // FP32 force: list records per staged tile (32 or 64; 0 = 32)
     int force_block;  // FP32 force: threads per block (256 or 128; 0 = 256)
     int32_t *item_cnt;
@@ -283,6 +283,7 @@ void nb_launch_build(nb_ctx *c, const double *pos, const float *mass, int64_t n)
 void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, int64_t n,
                              const int64_t *offsets, int64_t nsys);
 void nb_launch_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g);
+int nb_item_block(const nb_ctx *c);
 
 // nb_walk.cu
 int nb_walk_warps(nb_ctx *c);

@@ -1214,11 +1214,11 @@ k_group_scatter(const int32_t *__restrict__ gid, const int32_t *__restrict__ n_f
     }
 }
 
-// Force work items of a group of m members (iblock = 64: two targets per
-// lane, or 32): full items of iblock, then (iblock 64) one 32-target item
-// if more than 32 remain, then a tail of <= 32 targets, run as 32/m' source
-// streams with m' the tail rounded up to a power of two.  Word: first member
-// | log2(streams) << 27 | (1 << 30 for a 64-target item).
+// Force work items of a group of m members (iblock targets: 64, 32, 16 or
+// 8): full items of iblock, then (iblock 64) one 32-target item if more than
+// 32 remain, then a tail of fewer targets, m' of them with the tail rounded up
+// to a power of two.  Word: first member | ls << 27 (an item of 32 >> ls
+// targets) | (1 << 30 for a 64-target item).
 __device__ __forceinline__ int32_t item_count(int32_t m, int iblock)
 {
     int32_t c = m / iblock, rem = m - c * iblock;
@@ -1315,7 +1315,8 @@ k_items(const int32_t *__restrict__ item_off, const int32_t *__restrict__ gcount
         int32_t i0 = 0, k = 0;
         for (; m - i0 >= iblock; i0 += iblock, k++) {
             items[2 * (int64_t)(o + k)] = g;
-            items[2 * (int64_t)(o + k) + 1] = i0 | (iblock == 64 ? (1 << 30) : 0);
+            items[2 * (int64_t)(o + k) + 1] =
+                i0 | (iblock == 64 ? (1 << 30) : (__clz(iblock) - 26) << 27);
         }
         int32_t rem = m - i0;
         if (iblock == 64 && rem > 32) {
@@ -1352,8 +1353,29 @@ void nb_launch_group_theta(nb_ctx *c, const float *theta_g)
     nb_launched(c, "k_group_theta");
 }
 
+// Targets per force work item.  An item is one warp's work from start to end,
+// so with few particles large items leave most warps idle and the launch ends
+// with the longest list's item: 64 targets only where there are several items
+// for every resident warp.  Smaller items run as more source streams, which
+// costs more staging per interaction.  Measured (force pass, us, items of
+// 64 / 32 / 16 / 8 targets): 4096 Plummer 52 / 50 / 38 / 31; 16,384 halos
+// 142 / 94 / 67 / 55; 65,536 halos 224 / 142 / 89 / 76; 150,000 halos 214 /
+// 144 / 116 / 154; 500,000 halos 571 / 481 / 463 / 670 (quadrupole 1350 / 1155
+// / 1275 / 1451); 1M halos 1018 / 963 / 980 / 1452; 2M halos 1022 / 1022 /
+// 1065 / 1565.  The fused pass repeats its walk for every item, so 16 and 8
+// are taken only where it gains as well or loses little (16,384 halos 162 /
+// 135 / 122 / 167; 65,536 halos 270 / 234 / 282 / 425).  The choice depends on
+// the particle count alone: every path sums the same items in the same order.
+int nb_item_block(const nb_ctx *c)
+{
+    const int rows = c->item_rows * NB_WARP;
+    const int want = c->n <= 8192 ? 8 : c->n <= 32768 ? 16 : c->n <= 1500000 ? 32 : 64;
+    return want < rows ? want : rows;
+}
+
 void nb_launch_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g)
 {
+    const int iblock = nb_item_block(c);
     const int gcap = c->num_sms * 16;
     nb_launch(k_group_flags, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->n_count,
               c->n_parent, c->cnt, n_crit, c->gflag, c->err);
@@ -1364,12 +1386,12 @@ void nb_launch_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g)
               c->n_first, c->n_count, c->cnt, c->gnode, c->gfirst, c->gcount, c->n, c->err);
     nb_launched(c, "k_group_scatter");
     nb_launch(k_group_boxes, c->num_sms * 16, 256, 0, nb_queue(c), c->gfirst, c->gcount, c->p_hi,
-              c->cnt, theta, theta_g, c->gbox, c->item_cnt, c->item_rows * NB_WARP, c->n, c->err);
+              c->cnt, theta, theta_g, c->gbox, c->item_cnt, iblock, c->n, c->err);
     nb_launched(c, "k_group_boxes");
     nb_exclusive_scan(c, c->item_cnt, c->item_cnt, c->max_n, &c->cnt[CNT_GROUPS],
                       &c->cnt[CNT_ITEMS]);
     nb_launch(k_items, nb_grid(c->max_n, 256, gcap), 256, 0, nb_queue(c), c->item_cnt, c->gcount,
-              c->cnt, c->items, c->item_rows * NB_WARP, c->max_items, c->err);
+              c->cnt, c->items, iblock, c->max_items, c->err);
     nb_launched(c, "k_items");
 }
 
