@@ -316,7 +316,7 @@ k_force(const int32_t *__restrict__ items, const int32_t *__restrict__ order,
         if (lane == 0) it = (int)nb_atomic_add(&cnt[CNT_FORCE_Q], 1LL);
         it = __shfl_sync(FULL, it, 0);
         if (it >= nitems) break;
-        it = order[it];
+        if (order) it = order[it];
         if (it < 0 || it >= nitems) {
             if (lane == 0) nb_bad(cnt, err, SITE_FORCE, it);
             continue;
@@ -366,9 +366,9 @@ static void launch_force_t(nb_ctx *c, float eps2, float *acc, float *pot)
         if (blocks < 1) blocks = 1;
     }
     nb_launch(k_force<MODE, GUARD, TILE, BT, QUAD>, c->num_sms * blocks, BT, 0, nb_queue(c),
-              c->items, c->item_order, c->gfirst, c->gcount, c->glen, c->gbox, c->p_hi, c->p_lo,
-              c->perm, c->list_xm, c->list_q, c->list_cap, c->list_alloc, c->n, c->cnt, eps2, acc,
-              pot, c->err, c->max_items);
+              c->items, nb_small_system(c) ? nullptr : c->item_order, c->gfirst, c->gcount,
+              c->glen, c->gbox, c->p_hi, c->p_lo, c->perm, c->list_xm, c->list_q, c->list_cap,
+              c->list_alloc, c->n, c->cnt, eps2, acc, pot, c->err, c->max_items);
     nb_launched(c, QUAD ? "k_force (quadrupole)" : "k_force");
 }
 
@@ -392,14 +392,18 @@ static void launch_force(nb_ctx *c, float eps2, float *acc, float *pot)
 void nb_launch_forces(nb_ctx *c, float eps, float *acc, float *pot, int precision)
 {
     cudaMemsetAsync(&c->cnt[CNT_FORCE_Q], 0, sizeof(long long), c->stream);
-    cudaMemsetAsync(c->item_bkt, 0, sizeof(int32_t) * 2 * NB_IBKT, c->stream);
+    // (a small system's items all run at once, in any order)
+    const bool ordered = !nb_small_system(c);
     const int ig = c->num_sms * 2;
-    nb_launch(k_item_hist, ig, 256, 0, nb_queue(c), c->items, c->gcount, c->glen, c->cnt,
-              c->max_items, c->item_bkt);
-    nb_launched(c, "k_item_hist");
-    nb_launch(k_item_order, ig, 256, 0, nb_queue(c), c->items, c->gcount, c->glen, c->cnt,
-              c->max_items, c->item_bkt, c->item_order, c->err);
-    nb_launched(c, "k_item_order");
+    if (ordered) {
+        cudaMemsetAsync(c->item_bkt, 0, sizeof(int32_t) * 2 * NB_IBKT, c->stream);
+        nb_launch(k_item_hist, ig, 256, 0, nb_queue(c), c->items, c->gcount, c->glen, c->cnt,
+                  c->max_items, c->item_bkt);
+        nb_launched(c, "k_item_hist");
+        nb_launch(k_item_order, ig, 256, 0, nb_queue(c), c->items, c->gcount, c->glen, c->cnt,
+                  c->max_items, c->item_bkt, c->item_order, c->err);
+        nb_launched(c, "k_item_order");
+    }
     const float eps2 = eps * eps;
     const bool guard = !(eps2 >= FLT_MIN);
     if (c->quad && c->lists_quad) {   // FP32 and compensated modes (checked by the caller)

@@ -34,6 +34,7 @@
 #define NB_RS_TILE 4096   // keys per radix-sort tile (sizes the sort's per-tile buffers)
 #define NB_RS_TILE_MIN 3072   // the tile of the context's single-pass sort (nb_sort.cu)
 #define NB_DS_TILE 4096   // nodes per tile of the stable sort by depth
+#define NB_SMALL_N 8192   // particles of a system whose topology one block builds
 #define NB_EV_POOL 2048
 #define NB_IBLOCK 64   // targets per force work item (two per lane)
 #define NB_PROBE_THETA 1.2f  // opening angle of the feature probe walk
@@ -412,6 +413,12 @@ __device__ __forceinline__ void nb_grid_wait()
 }
 
 #define NB_OVERLAP_MAX_N 2500000
+
+// one system that one block's topology and groups cover
+static inline bool nb_small_system(const nb_ctx *c)
+{
+    return c->nsys == 1 && c->n <= NB_SMALL_N;
+}
 
 // a stream and whether launches on it overlap
 struct nb_queue {

@@ -941,6 +941,7 @@ k_moments(const int32_t *__restrict__ clist, int64_t clist_len, nb_wrec *__restr
 
 static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t n,
                        const int32_t *sys_sorted);
+static void launch_topology_small(nb_ctx *c, int64_t n);
 
 void nb_launch_build(nb_ctx *c, const double *pos, const float *mass, int64_t n)
 {
@@ -952,7 +953,8 @@ void nb_launch_build(nb_ctx *c, const double *pos, const float *mass, int64_t n)
     nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(c), pos, n, c->root, nullptr, c->keys,
               c->idx, c->key_order);
     nb_launched(c, "k_keys");
-    nb_radix_sort(c, n);
+    if (nb_small_system(c)) launch_topology_small(c, n);
+    else nb_radix_sort(c, n);
     build_tail(c, pos, mass, n, nullptr);
 }
 
@@ -1115,13 +1117,9 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
     nb_launched(c, "k_sys_roots");
 }
 
-static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t n,
-                       const int32_t *sys_sorted)
+// cells, parents and the level order of the sorted particles
+static void topology(nb_ctx *c, int64_t n, const int32_t *sys_sorted, int gcap)
 {
-    cudaStream_t s = c->stream;
-    nb_launch(k_gather, nb_grid(n, 256), 256, 0, nb_queue(c), pos, mass, n, c->idx, c->perm,
-              c->p_x64, c->p_hi, c->p_lo, c->cnt, c->err);
-    nb_launched(c, "k_gather");
     nb_launch(k_levels, nb_grid(n, 256), 256, 0, nb_queue(c), c->keys, n, sys_sorted, c->clev,
               c->ccount);
     nb_launched(c, "k_levels");
@@ -1130,7 +1128,6 @@ static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t 
               c->node_c, c->n_level, c->n_first, c->n_count, c->n_parent, c->n_nchild, c->n_depth,
               c->cnt, sys_sorted, c->sys_off, c->err);
     nb_launched(c, "k_cells");
-    const int gcap = c->num_sms * 16;
     nb_launch(k_cell_ends, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->keys, n,
               c->cstart, c->n_level, c->n_first, c->node_c, c->n_count, c->cnt, sys_sorted,
               c->sys_off, c->err);
@@ -1149,6 +1146,17 @@ static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t 
     nb_launched(c, "k_depth_scatter");
     nb_launch(k_level_start, 1, 32, 0, nb_queue(c), c->dhist, nt, c->level_start);
     nb_launched(c, "k_level_start");
+}
+
+static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t n,
+                       const int32_t *sys_sorted)
+{
+    cudaStream_t s = c->stream;
+    nb_launch(k_gather, nb_grid(n, 256), 256, 0, nb_queue(c), pos, mass, n, c->idx, c->perm,
+              c->p_x64, c->p_hi, c->p_lo, c->cnt, c->err);
+    nb_launched(c, "k_gather");
+    const int gcap = c->num_sms * 16;
+    if (!nb_small_system(c)) topology(c, n, sys_sorted, gcap);
     cudaMemsetAsync(c->cbkt_cnt, 0, sizeof(int32_t) * 2 * NB_CBKT, s);
     nb_launch(k_bfs_records, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->bfs2pid,
               c->pid2bfs, c->node_c, c->n_first, c->n_nchild, c->n_parent, c->n_depth, c->keys,
@@ -1226,6 +1234,15 @@ __device__ __forceinline__ int32_t item_count(int32_t m, int iblock)
     return c + (rem > 0 ? 1 : 0);
 }
 
+// centre of a group's box and 1/theta, rounded to FP32
+__device__ __forceinline__ float4 group_centre(const float4 &lo, const float4 &hi, float th)
+{
+    return make_float4(__double2float_rn(__dmul_rn(0.5, __dadd_rn((double)lo.x, (double)hi.x))),
+                       __double2float_rn(__dmul_rn(0.5, __dadd_rn((double)lo.y, (double)hi.y))),
+                       __double2float_rn(__dmul_rn(0.5, __dadd_rn((double)lo.z, (double)hi.z))),
+                       __double2float_rn(__ddiv_rn(1.0, (double)th)));
+}
+
 // group box over the members' FP32 positions, its FP32 centre, FP32
 // 1/theta, and the number of force work items of the group.  A warp takes GB
 // consecutive groups: for each in turn the members are strided over the lanes
@@ -1287,15 +1304,36 @@ k_group_boxes(const int32_t *__restrict__ gfirst, const int32_t *__restrict__ gc
             item_cnt[gl] = 0;
             continue;
         }
-        const float th = theta_g ? theta_g[gl] : theta;
-        const float invth = __double2float_rn(__ddiv_rn(1.0, (double)th));
-        const float cx = __double2float_rn(__dmul_rn(0.5, __dadd_rn((double)blx, (double)bhx)));
-        const float cy = __double2float_rn(__dmul_rn(0.5, __dadd_rn((double)bly, (double)bhy)));
-        const float cz = __double2float_rn(__dmul_rn(0.5, __dadd_rn((double)blz, (double)bhz)));
-        gbox[3 * (int64_t)gl] = make_float4(blx, bly, blz, 0.0f);
-        gbox[3 * (int64_t)gl + 1] = make_float4(bhx, bhy, bhz, 0.0f);
-        gbox[3 * (int64_t)gl + 2] = make_float4(cx, cy, cz, invth);
+        const float4 lo = make_float4(blx, bly, blz, 0.0f), hi = make_float4(bhx, bhy, bhz, 0.0f);
+        gbox[3 * (int64_t)gl] = lo;
+        gbox[3 * (int64_t)gl + 1] = hi;
+        gbox[3 * (int64_t)gl + 2] = group_centre(lo, hi, theta_g ? theta_g[gl] : theta);
         item_cnt[gl] = item_count(ml, iblock);
+    }
+}
+
+// the work items of group g (m members) at items o, o + 1, ...
+__device__ __forceinline__ void put_items(int32_t *items, int32_t o, int32_t g, int32_t m,
+                                          int iblock)
+{
+    int32_t i0 = 0, k = 0;
+    for (; m - i0 >= iblock; i0 += iblock, k++) {
+        items[2 * (int64_t)(o + k)] = g;
+        items[2 * (int64_t)(o + k) + 1] =
+            i0 | (iblock == 64 ? (1 << 30) : (__clz(iblock) - 26) << 27);
+    }
+    int32_t rem = m - i0;
+    if (iblock == 64 && rem > 32) {
+        items[2 * (int64_t)(o + k)] = g;
+        items[2 * (int64_t)(o + k) + 1] = i0;
+        i0 += 32;
+        rem -= 32;
+        k++;
+    }
+    if (rem > 0) {
+        const int lg = rem > 1 ? 32 - __clz(rem - 1) : 0;   // log2 of rem rounded up
+        items[2 * (int64_t)(o + k)] = g;
+        items[2 * (int64_t)(o + k) + 1] = i0 | ((5 - lg) << 27);
     }
 }
 
@@ -1312,25 +1350,7 @@ k_items(const int32_t *__restrict__ item_off, const int32_t *__restrict__ gcount
         if (!nb_in(o >= 0 && (int64_t)o + item_count(m, iblock) <= max_items, cnt, err,
                    SITE_ITEMS, g))
             continue;
-        int32_t i0 = 0, k = 0;
-        for (; m - i0 >= iblock; i0 += iblock, k++) {
-            items[2 * (int64_t)(o + k)] = g;
-            items[2 * (int64_t)(o + k) + 1] =
-                i0 | (iblock == 64 ? (1 << 30) : (__clz(iblock) - 26) << 27);
-        }
-        int32_t rem = m - i0;
-        if (iblock == 64 && rem > 32) {
-            items[2 * (int64_t)(o + k)] = g;
-            items[2 * (int64_t)(o + k) + 1] = i0;
-            i0 += 32;
-            rem -= 32;
-            k++;
-        }
-        if (rem > 0) {
-            const int lg = rem > 1 ? 32 - __clz(rem - 1) : 0;   // log2 of rem rounded up
-            items[2 * (int64_t)(o + k)] = g;
-            items[2 * (int64_t)(o + k) + 1] = i0 | ((5 - lg) << 27);
-        }
+        put_items(items, o, g, m, iblock);
     }
 }
 
@@ -1351,6 +1371,375 @@ void nb_launch_group_theta(nb_ctx *c, const float *theta_g)
     nb_launch(k_group_theta, nb_grid(c->max_n, 256, c->num_sms * 8), 256, 0, nb_queue(c), theta_g,
               c->cnt, c->gbox);
     nb_launched(c, "k_group_theta");
+}
+
+// ------------------------------------------------------------ small systems
+// Up to NB_SMALL_N particles of one system: everything between the keys and
+// the node records that needs no FP64 in one block, and the groups in
+// another.  The launches they replace (21 and 8) do a microsecond of work
+// each at these sizes and cost four to five from start to start; one block
+// pays a barrier instead.  The keys, records and moments stay spread over the
+// device: FP64 runs at 2 lanes per clock on an SM.  Measured (build / groups
+// and walk, us, in a captured step, separate launches and so): 1000 uniform
+// particles 125 / 60 and 87 / 53, 4096 Plummer 160 / 77 and 146 / 80; an eager
+// force evaluation 266 and 201, 351 and 301.
+// The results are those of the separate launches, element for element.
+#define SM_T 1024
+#define SM_W (SM_T / NB_WARP)
+#define SM_I (NB_SMALL_N / SM_T)   // keys per thread at most
+
+struct SmallSmem {
+    uint64_t key[NB_SMALL_N];
+    int32_t idx[NB_SMALL_N + 1];    // sorted order; then the scanned cell counts
+    uint32_t hist[SM_W][256];
+    uint32_t start[256];
+    int32_t wsum[SM_W];
+    int8_t clev[NB_SMALL_N];
+};
+
+// exclusive scan of one value per thread over the block; *total gets the sum
+__device__ __forceinline__ int32_t small_scan(int32_t v, int32_t *wsum, int32_t *total)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();   // wsum is free
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    int32_t t = wsum[lane], p = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, p, o);
+        if (lane >= o) p += y;
+    }
+    *total = __shfl_sync(0xffffffffu, p, 31);
+    const int32_t before = w > 0 ? __shfl_sync(0xffffffffu, p, w > 0 ? w - 1 : 0) : 0;
+    return before + x - v;
+}
+
+// Sort of (key, index), cells, their ends, parents and children, and the
+// level order.  Pointers written here are read here again: no read-only
+// loads (no const __restrict__) on them.
+__global__ void __launch_bounds__(SM_T, 1)
+k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t *n_level,
+                 int32_t *n_first, int32_t *n_count, int32_t *n_parent, int32_t *n_nchild,
+                 int8_t *n_depth, int32_t *bfs2pid, int32_t *pid2bfs, int32_t *level_start,
+                 int32_t *arrive, int32_t *lcount, long long *cnt, unsigned *err)
+{
+    nb_grid_wait();
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    SmallSmem &S = *reinterpret_cast<SmallSmem *>(sm_raw);
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int I = (n + SM_T - 1) / SM_T;   // keys per thread
+
+    // stable LSD radix sort, 8-bit digits: a warp holds I rounds of 32
+    // consecutive keys in registers, ranks them round by round (ballot match,
+    // running counts) and writes them back to shared memory in digit order
+    uint64_t k[SM_I];
+    uint32_t v[SM_I];
+    int e[SM_I];
+#pragma unroll
+    for (int r = 0; r < SM_I; r++) {
+        e[r] = r < I ? (w * I + r) * NB_WARP + lane : n;
+        k[r] = e[r] < n ? key[e[r]] : 0ull;
+        v[r] = (uint32_t)e[r];
+    }
+    for (int shift = 0; shift < 64; shift += 8) {
+        for (int i = tid; i < SM_W * 256; i += SM_T) (&S.hist[0][0])[i] = 0u;
+        __syncthreads();
+        uint32_t rnk[SM_I];
+#pragma unroll
+        for (int r = 0; r < SM_I; r++) {
+            if (r >= I) break;
+            const bool ok = e[r] < n;
+            const int d = (int)((k[r] >> shift) & 255u);
+            const unsigned peers = nb_match_bits<8>((unsigned)d, ok);
+            const unsigned before = __popc(peers & lt);
+            const uint32_t pre = ok ? S.hist[w][d] : 0u;
+            __syncwarp();
+            if (ok && before == 0) S.hist[w][d] = pre + __popc(peers);
+            __syncwarp();
+            rnk[r] = pre + before;
+        }
+        __syncthreads();
+        int32_t run = 0;
+        if (tid < 256)
+#pragma unroll 8
+            for (int ww = 0; ww < SM_W; ww++) {
+                const uint32_t c = S.hist[ww][tid];
+                S.hist[ww][tid] = (uint32_t)run;
+                run += (int32_t)c;
+            }
+        int32_t all;
+        const int32_t st = small_scan(run, S.wsum, &all);
+        if (tid < 256) S.start[tid] = (uint32_t)st;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < SM_I; r++)
+            if (e[r] < n) {
+                const int d = (int)((k[r] >> shift) & 255u);
+                const uint32_t pos = S.start[d] + S.hist[w][d] + rnk[r];
+                if (!nb_in(pos < (uint32_t)n, cnt, err, SITE_SORT, pos)) continue;
+                S.key[pos] = k[r];
+                S.idx[pos] = (int32_t)v[r];
+            }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < SM_I; r++)
+            if (e[r] < n) {
+                k[r] = S.key[e[r]];
+                v[r] = (uint32_t)S.idx[e[r]];
+            }
+    }
+#pragma unroll
+    for (int r = 0; r < SM_I; r++)
+        if (e[r] < n) {
+            key[e[r]] = k[r];
+            idx[e[r]] = v[r];
+        }
+
+    // cells per particle, scanned (a thread's I consecutive particles)
+    int32_t cc[SM_I], mine = 0;
+#pragma unroll
+    for (int r = 0; r < SM_I; r++) {
+        const int a = tid * I + r;
+        cc[r] = 0;
+        if (r < I && a < n) {
+            const int ca = a + 1 < n ? common_levels(S.key[a], S.key[a + 1]) : -1;
+            const int cp = a > 0 ? common_levels(S.key[a - 1], S.key[a]) : -1;
+            S.clev[a] = (int8_t)ca;
+            cc[r] = ca > cp ? ca - cp : 0;
+        }
+        mine += cc[r];
+    }
+    int32_t C;
+    int32_t at = small_scan(mine, S.wsum, &C);   // (its barriers: idx is read)
+    int32_t *cst = S.idx;
+#pragma unroll
+    for (int r = 0; r < SM_I; r++) {
+        const int a = tid * I + r;
+        if (r < I && a < n) cst[a] = at;
+        at += cc[r];
+    }
+    if (tid == 0) {
+        cst[n] = C;
+        cnt[CNT_CELLS] = C;
+    }
+    __syncthreads();
+    const int32_t total = C + n;
+
+    // nodes: leaves and cells by their first particle, and the cells' ends
+    int deepest = -1;
+    for (int a = tid; a < n; a += SM_T) {
+        deepest = max(deepest, cell_records(a, n, S.clev, cst, node_c, n_level, n_first, n_count,
+                                            n_parent, n_nchild, n_depth, cnt, err));
+        const int ca = S.clev[a], cp = a > 0 ? S.clev[a - 1] : -1;
+        const int32_t base = cst[a] + a;
+        for (int lev = ca; lev > cp; lev--) {
+            const int shift = 63 - 3 * lev;
+            const uint64_t P = S.key[a] >> shift;
+            int lo = a, step = 1, hi = a + 1;
+            while (hi < n && (S.key[hi] >> shift) == P) {
+                lo = hi;
+                step <<= 1;
+                hi = lo + step;
+            }
+            if (hi > n) hi = n;
+            while (hi - lo > 1) {
+                const int mid = lo + ((hi - lo) >> 1);
+                if ((S.key[mid] >> shift) == P) lo = mid;
+                else hi = mid;
+            }
+            const int32_t id = base + (lev - cp - 1);
+            node_c[id] = make_int4(cst[lo + 1] + lo + 1, 0, 0, 0);
+            n_count[id] = lo - a + 1;
+        }
+    }
+    deepest = __reduce_max_sync(FULL, deepest);
+    if (lane == 0 && deepest >= 0) atomicMax(&cnt[CNT_MAXLEVEL], (long long)deepest);
+    for (int i = tid; i < SM_W * 32; i += SM_T) (&S.hist[0][0])[i] = 0u;
+    __syncthreads();
+
+    // parents and child counts; nodes per depth in each warp's run of nodes
+    uint32_t(*dh)[32] = reinterpret_cast<uint32_t(*)[32]>(&S.hist[0][0]);
+    const int32_t per = ((total + SM_T - 1) / SM_T) * NB_WARP;   // nodes of a warp
+    const int32_t u0 = w * per, u1 = min(u0 + per, total);
+    for (int32_t ub = u0; ub < u1; ub += NB_WARP) {
+        const int32_t u = ub + lane;
+        const bool ok = u < u1;
+        if (ok) {
+            arrive[u] = 0;
+            lcount[u] = 0;
+            const int4 cu = node_c[u];
+            if (!cu.w && nb_in(cu.x <= total, cnt, err, SITE_PARENTS, cu.x)) {
+                int32_t ch = u + 1, nch = 0;
+                while (ch < cu.x) {
+                    n_parent[ch] = u;
+                    nch++;
+                    const int32_t nx = node_c[ch].x;
+                    ch = nx > ch ? nx : cu.x;   // next always advances
+                }
+                n_nchild[u] = nch;
+            }
+        }
+        const int d = ok ? (int)n_depth[u] : 0;
+        const bool in = ok && nb_in(d >= 0 && d < NB_DEPTHS, cnt, err, SITE_DEPTH, u);
+        const unsigned peers = nb_match_bits<5>((unsigned)d & 31u, in);
+        if (in && (peers & lt) == 0) dh[w][d] += __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    if (w == 0) {   // lane d: its depth's counts over the warps, then over the depths
+        uint32_t run = 0;
+        for (int ww = 0; ww < SM_W; ww++) {
+            const uint32_t c = dh[ww][lane];
+            dh[ww][lane] = run;
+            run += c;
+        }
+        uint32_t x = run;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        S.start[lane] = x - run;
+        if (lane <= NB_DEPTHS) level_start[lane] = (int32_t)(x - run);
+    }
+    __syncthreads();
+    // level order, stable: preorder inside a depth
+    for (int32_t ub = u0; ub < u1; ub += NB_WARP) {
+        const int32_t u = ub + lane;
+        const int d = u < u1 ? (int)n_depth[u] : 0;
+        const bool in = u < u1 && d >= 0 && d < NB_DEPTHS;
+        const unsigned peers = nb_match_bits<5>((unsigned)d & 31u, in);
+        const uint32_t pre = in ? dh[w][d] : 0u;
+        __syncwarp();
+        if (in && (peers & lt) == 0) dh[w][d] = pre + __popc(peers);
+        __syncwarp();
+        if (!in) continue;
+        const int32_t b = (int32_t)(S.start[d] + pre + __popc(peers & lt));
+        if (!nb_in(b < total, cnt, err, SITE_DEPTH, b)) continue;
+        bfs2pid[b] = u;
+        pid2bfs[u] = b;
+    }
+}
+
+// Groups, their boxes and centres, and the force work items (the launches
+// of nb_launch_groups).
+__global__ void __launch_bounds__(SM_T, 1)
+k_groups_small(const int32_t *__restrict__ n_count, const int32_t *__restrict__ n_parent,
+               const int32_t *__restrict__ n_first, const float4 *__restrict__ p_hi,
+               long long *cnt, int n_crit, float theta, const float *__restrict__ theta_g,
+               int32_t *gnode, int32_t *gfirst, int32_t *gcount, float4 *gbox, int32_t *items,
+               int iblock, int64_t max_items, int32_t n, unsigned *err)
+{
+    nb_grid_wait();
+    __shared__ int32_t wsum[SM_W];
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int32_t total = (int32_t)cnt[CNT_NODES];
+    // group ids in preorder: a warp takes a run of nodes, 32 at a time
+    const int32_t per = ((total + SM_T - 1) / SM_T) * NB_WARP;
+    const int32_t u0 = w * per, u1 = min(u0 + per, total);
+    auto flag = [&](int32_t u) -> bool {
+        if (u >= u1) return false;
+        const int32_t p = n_parent[u];
+        return n_count[u] <= n_crit && (p < 0 || p >= total || n_count[p] > n_crit);
+    };
+    int32_t found = 0;
+    for (int32_t ub = u0; ub < u1; ub += NB_WARP) {
+        const int32_t u = ub + lane;
+        if (u < u1) nb_in(n_parent[u] < total, cnt, err, SITE_GROUPS, u);
+        found += __popc(__ballot_sync(FULL, flag(u)));
+    }
+    int32_t G;
+    int32_t at = small_scan(lane == 0 ? found : 0, wsum, &G);
+    at = __shfl_sync(FULL, at, 0);
+    for (int32_t ub = u0; ub < u1; ub += NB_WARP) {
+        const int32_t u = ub + lane;
+        const bool is = flag(u);
+        const unsigned m = __ballot_sync(FULL, is);
+        const int32_t g = at + __popc(m & ((1u << lane) - 1u));
+        at += __popc(m);
+        if (is && nb_in(g < n, cnt, err, SITE_GROUPS, g)) {
+            gnode[g] = u;
+            gfirst[g] = n_first[u];
+            gcount[g] = n_count[u];
+        }
+    }
+    if (tid == 0) cnt[CNT_GROUPS] = G;
+    __syncthreads();
+    // boxes over the members' FP32 positions, a warp per group
+    for (int32_t g = w; g < G; g += SM_W) {
+        const int32_t f = gfirst[g], m = gcount[g];
+        if (!(f >= 0 && m >= 1 && f + m <= n)) {
+            if (lane == 0) nb_bad(cnt, err, SITE_GROUPS, g);
+            continue;
+        }
+        float lx = INFINITY, ly = INFINITY, lz = INFINITY;
+        float hx = -INFINITY, hy = -INFINITY, hz = -INFINITY;
+        for (int32_t j = lane; j < m; j += NB_WARP) {
+            const float4 p = p_hi[f + j];
+            lx = fminf(lx, p.x); ly = fminf(ly, p.y); lz = fminf(lz, p.z);
+            hx = fmaxf(hx, p.x); hy = fmaxf(hy, p.y); hz = fmaxf(hz, p.z);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lx = fminf(lx, __shfl_xor_sync(FULL, lx, o));
+            ly = fminf(ly, __shfl_xor_sync(FULL, ly, o));
+            lz = fminf(lz, __shfl_xor_sync(FULL, lz, o));
+            hx = fmaxf(hx, __shfl_xor_sync(FULL, hx, o));
+            hy = fmaxf(hy, __shfl_xor_sync(FULL, hy, o));
+            hz = fmaxf(hz, __shfl_xor_sync(FULL, hz, o));
+        }
+        if (lane == 0) {
+            gbox[3 * g] = make_float4(lx, ly, lz, 0.0f);
+            gbox[3 * g + 1] = make_float4(hx, hy, hz, 0.0f);
+        }
+    }
+    __syncthreads();
+    // centres and 1/theta, a lane per group, and the work items in group order
+    int32_t done = 0;
+    for (int32_t g0 = 0; g0 < G; g0 += SM_T) {
+        const int32_t g = g0 + tid;
+        int32_t m = 0;
+        if (g < G) {
+            const int32_t f = gfirst[g];
+            m = gcount[g];
+            if (!(f >= 0 && m >= 1 && f + m <= n)) m = 0;   // (reported above)
+        }
+        if (m > 0) {
+            const float4 lo = gbox[3 * g], hi = gbox[3 * g + 1];
+            const float th = theta_g ? theta_g[g] : theta;
+            gbox[3 * g + 2] = group_centre(lo, hi, th);
+        }
+        int32_t all;
+        const int32_t o = done + small_scan(m > 0 ? item_count(m, iblock) : 0, wsum, &all);
+        done += all;
+        if (m > 0 && nb_in((int64_t)o + item_count(m, iblock) <= max_items, cnt, err, SITE_ITEMS, g))
+            put_items(items, o, g, m, iblock);
+    }
+    if (tid == 0) cnt[CNT_ITEMS] = done;
+}
+
+static void launch_topology_small(nb_ctx *c, int64_t n)
+{
+    static bool done = false;
+    if (!done) {
+        cudaFuncSetAttribute(k_topology_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(SmallSmem));
+        done = true;
+    }
+    nb_launch(k_topology_small, 1, SM_T, sizeof(SmallSmem), nb_queue(c), c->keys, c->idx, (int)n,
+              c->node_c, c->n_level, c->n_first, c->n_count, c->n_parent, c->n_nchild, c->n_depth,
+              c->bfs2pid, c->pid2bfs, c->level_start, c->arrive, c->lcount, c->cnt, c->err);
+    nb_launched(c, "k_topology_small");
 }
 
 // Targets per force work item.  An item is one warp's work from start to end,
@@ -1376,6 +1765,13 @@ int nb_item_block(const nb_ctx *c)
 void nb_launch_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g)
 {
     const int iblock = nb_item_block(c);
+    if (nb_small_system(c)) {
+        nb_launch(k_groups_small, 1, SM_T, 0, nb_queue(c), c->n_count, c->n_parent, c->n_first,
+                  c->p_hi, c->cnt, n_crit, theta, theta_g, c->gnode, c->gfirst, c->gcount, c->gbox,
+                  c->items, iblock, c->max_items, (int)c->n, c->err);
+        nb_launched(c, "k_groups_small");
+        return;
+    }
     const int gcap = c->num_sms * 16;
     nb_launch(k_group_flags, nb_grid(c->max_nodes, 256, gcap), 256, 0, nb_queue(c), c->n_count,
               c->n_parent, c->cnt, n_crit, c->gflag, c->err);

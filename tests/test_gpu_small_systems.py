@@ -1,19 +1,49 @@
-"""Sizes where the force work items change: they hold 8 targets up to 8192
-particles, 16 up to 32,768, then 32.  On both sides of a line forces meet the
-tolerances of the parity tests, and the fused and overlapped passes sum the
-same items in the same order (the same bits).
+"""Sizes where the launches and the force work items change: one block builds
+the topology and the groups up to 8192 particles (1024 threads), items hold 8
+targets up to 8192 particles, 16 up to 32,768, then 32.  Trees, groups and
+lists must equal the oracle's bit for bit on both sides of every line, forces
+meet the tolerances of the parity tests, and the fused and overlapped passes
+sum the same items in the same order (the same bits).
 """
 import numpy as np
 import pytest
 
 import nbsynth
 from tests.gpu_common import gpu_run
+from tests.test_gpu_parity import assert_lists_equal, assert_tree_equal, clump_set
 
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
+
+
+@pytest.mark.parametrize("order", ["morton", "hilbert"])
+@pytest.mark.parametrize("n,n_crit", [(1, 1), (2, 1), (33, 8), (1023, 32), (1024, 1), (1025, 64),
+                                      (5000, 8192), (8191, 17), (8192, 64), (8193, 64)])
+def test_tree_groups_lists(oracle_lib, n, n_crit, order):
+    ps = nbsynth.halo_mix(n, 60 + n, n_halos=5) if n > 100 else nbsynth.plummer(n, 60 + n)
+    g = gpu_run(ps.pos, ps.mass, theta=0.7, n_crit=n_crit, eps=1e-3, key_order=order)
+    T = oracle_lib.Tree(ps.pos, ps.mass, order=order)
+    assert_tree_equal(g, T)
+    if n_crit > 1 or n < 100:
+        assert_lists_equal(g, T, 0.7, n_crit)
+
+
+@pytest.mark.parametrize("n", [4000, 8192])
+def test_deep_chains_and_coincident_points(oracle_lib, n):
+    """Pairs 1e-6 apart and coincident points: cells down to the last level,
+    several nodes per particle."""
+    rng = np.random.default_rng(n)
+    pos, mass = clump_set(n, n)
+    k = n // 3
+    pos[:k] = pos[k:2 * k] + 1e-6 * rng.normal(size=(k, 3))
+    pos[5:25] = pos[4]
+    g = gpu_run(pos, mass, theta=0.6, n_crit=16, eps=1e-3)
+    T = oracle_lib.Tree(pos, mass)
+    assert_tree_equal(g, T)
+    assert_lists_equal(g, T, 0.6, 16)
 
 
 @pytest.mark.parametrize("n", [8192, 8193, 32768, 32769])
