@@ -282,6 +282,14 @@ static int sync_read(nb_ctx *c)
     return rc ? rc : err_code(bits);
 }
 
+// the error word and the counters with one synchronisation
+static int sync_read_all(nb_ctx *c, unsigned *bits)
+{
+    CK(cudaMemcpyAsync(c->cnt_host, c->cnt, sizeof(long long) * CNT_N_, cudaMemcpyDeviceToHost,
+                       c->stream));
+    return sync_read_bits(c, bits);
+}
+
 static int read_counters(nb_ctx *c)
 {
     CK(cudaMemcpyAsync(c->cnt_host, c->cnt, sizeof(long long) * CNT_N_,
@@ -528,6 +536,26 @@ static int walk_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g,
     if (formed) nb_launch_group_theta(c, theta_g);
     else nb_launch_groups(c, theta, n_crit, theta_g);
     c->has_groups = 1;
+    if (c->sync_checks && c->list_alloc > 0 && c->list_cap > 0 && c->wq &&
+        !(c->quad && !c->list_q)) {
+        // storage from an earlier walk: walk at once, without waiting for the
+        // number of groups (the walk stays inside the storage and reports
+        // what does not fit; the loop below then sizes it and walks again)
+        nb_launch_walk(c);
+        if (cudaGetLastError() != cudaSuccess) return NB_ERR_CUDA;
+        unsigned bits = 0;
+        int rc = sync_read_all(c, &bits);
+        if (rc) return rc;
+        c->groups_host = c->cnt_host[CNT_GROUPS];
+        rc = err_code(bits);
+        if (rc != NB_ERR_CAPACITY) {
+            phase_end(c, tk, NB_PHASE_WALK);
+            if (rc) return rc;
+            c->has_lists = 1;
+            c->lists_quad = c->quad;
+            return NB_OK;
+        }
+    }
     if (c->sync_checks) {
         int rc = read_counters(c);
         if (rc) return rc;

@@ -843,19 +843,34 @@ __device__ __forceinline__ void cell_quad(int32_t b, int4 wb, const double com[3
                                           const double *b_mass, const double *b_com, double *b_q)
 {
     double q[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int32_t k = 0; k < wb.w; k++) {
-        const int64_t c = (int64_t)wb.z + k;
-        const double m = __ldcg(&b_mass[c]);
-        double d[3];
+    // the loads of QB children at a time are in flight together: the fold is
+    // on the path from the deepest cells to the root, one level after another
+    constexpr int QB = 4;
+    for (int32_t k0 = 0; k0 < wb.w; k0 += QB) {
+        double m[QB], x[QB][3], cq[QB][6];
 #pragma unroll
-        for (int a = 0; a < 3; a++) d[a] = __ldcg(&b_com[3 * c + a]) - com[a];
-        const double d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-        q[0] += __ldcg(&b_q[6 * c + 0]) + m * (3.0 * d[0] * d[0] - d2);
-        q[1] += __ldcg(&b_q[6 * c + 1]) + m * (3.0 * d[1] * d[1] - d2);
-        q[2] += __ldcg(&b_q[6 * c + 2]) + m * (3.0 * d[2] * d[2] - d2);
-        q[3] += __ldcg(&b_q[6 * c + 3]) + m * 3.0 * d[0] * d[1];
-        q[4] += __ldcg(&b_q[6 * c + 4]) + m * 3.0 * d[0] * d[2];
-        q[5] += __ldcg(&b_q[6 * c + 5]) + m * 3.0 * d[1] * d[2];
+        for (int k = 0; k < QB; k++) {
+            const int64_t c = (int64_t)wb.z + (k0 + k < wb.w ? k0 + k : wb.w - 1);
+            m[k] = __ldcg(&b_mass[c]);
+#pragma unroll
+            for (int a = 0; a < 3; a++) x[k][a] = __ldcg(&b_com[3 * c + a]);
+#pragma unroll
+            for (int a = 0; a < 6; a++) cq[k][a] = __ldcg(&b_q[6 * c + a]);
+        }
+#pragma unroll
+        for (int k = 0; k < QB; k++) {
+            if (k0 + k >= wb.w) break;
+            double d[3];
+#pragma unroll
+            for (int a = 0; a < 3; a++) d[a] = x[k][a] - com[a];
+            const double d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+            q[0] += cq[k][0] + m[k] * (3.0 * d[0] * d[0] - d2);
+            q[1] += cq[k][1] + m[k] * (3.0 * d[1] * d[1] - d2);
+            q[2] += cq[k][2] + m[k] * (3.0 * d[2] * d[2] - d2);
+            q[3] += cq[k][3] + m[k] * 3.0 * d[0] * d[1];
+            q[4] += cq[k][4] + m[k] * 3.0 * d[0] * d[2];
+            q[5] += cq[k][5] + m[k] * 3.0 * d[1] * d[2];
+        }
     }
 #pragma unroll
     for (int k = 0; k < 6; k++) b_q[6 * (int64_t)b + k] = q[k];
