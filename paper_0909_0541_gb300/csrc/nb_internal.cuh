@@ -34,7 +34,7 @@
 #define NB_RS_TILE 4096   // keys per radix-sort tile (sizes the sort's per-tile buffers)
 #define NB_RS_TILE_MIN 3072   // the tile of the context's single-pass sort (nb_sort.cu)
 #define NB_DS_TILE 4096   // nodes per tile of the stable sort by depth
-#define NB_SMALL_N 8192   // particles of a system whose topology one block builds
+#define NB_SMALL_N 4096   // particles of a system whose topology one block builds
 #define NB_EV_POOL 2048
 #define NB_IBLOCK 64   // targets per force work item (two per lane)
 #define NB_PROBE_THETA 1.2f  // opening angle of the feature probe walk
@@ -399,11 +399,12 @@ static __device__ __forceinline__ int32_t nb_block_scan256(int32_t v, int32_t *t
 // is a chain of about 40 dependent kernels, and below some 100,000 particles
 // the gaps between them were a third of its time (build, walk and force with
 // plain launches and with these: 355 -> 274 us at 1000 particles, 513 -> 427
-// at 16,384, 1343 -> 1276 at 500,000, 2593 -> 2491 at 2.1M).  In large steps
-// the gaps no longer show and the early blocks cost more than they save (two
-// captured steps of 7.66M particles in 512 systems: 21.06 ms with plain
-// launches, 21.66 with these; of 2.87M the same either way), so launches
-// overlap up to NB_OVERLAP_MAX_N particles.  Every kernel of the chain calls
+// at 16,384, 1343 -> 1276 at 500,000, 2593 -> 2491 at 2.1M).  A captured
+// graph's gaps are shorter (a step of 16,384: 389 -> 370 us, of 65,536 533 ->
+// 494, of 500,000 1222 -> 1227), and in large steps the early blocks cost more
+// than the gaps (1.93M particles 4.27 -> 4.47 ms; 7.66M in 512 systems 10.53
+// -> 10.83).  So launches overlap up to NB_OVERLAP_MAX_N particles, in a
+// capture up to NB_OVERLAP_GRAPH_MAX_N.  Every kernel of the chain calls
 // nb_grid_wait first, in every thread: what comes before it is then complete,
 // and through it all earlier launches.
 __device__ __forceinline__ void nb_grid_wait()
@@ -413,6 +414,7 @@ __device__ __forceinline__ void nb_grid_wait()
 }
 
 #define NB_OVERLAP_MAX_N 2500000
+#define NB_OVERLAP_GRAPH_MAX_N 200000
 
 // one system that one block's topology and groups cover
 static inline bool nb_small_system(const nb_ctx *c)
@@ -425,7 +427,9 @@ struct nb_queue {
     cudaStream_t stream;
     bool overlap;
     nb_queue(cudaStream_t s, int64_t n) : stream(s), overlap(n <= NB_OVERLAP_MAX_N) {}
-    explicit nb_queue(const nb_ctx *c) : nb_queue(c->stream, c->n) {}
+    explicit nb_queue(const nb_ctx *c)
+        : stream(c->stream),
+          overlap(c->n <= (c->capturing ? NB_OVERLAP_GRAPH_MAX_N : NB_OVERLAP_MAX_N)) {}
 };
 
 template <typename... P, typename... A>

@@ -1394,20 +1394,22 @@ void nb_launch_group_theta(nb_ctx *c, const float *theta_g)
 // another.  The launches they replace (21 and 8) do a microsecond of work
 // each at these sizes and cost four to five from start to start; one block
 // pays a barrier instead.  The keys, records and moments stay spread over the
-// device: FP64 runs at 2 lanes per clock on an SM.  Measured (build / groups
-// and walk, us, in a captured step, separate launches and so): 1000 uniform
-// particles 125 / 60 and 87 / 53, 4096 Plummer 160 / 77 and 146 / 80; an eager
-// force evaluation 266 and 201, 351 and 301.
+// device: FP64 runs at 2 lanes per clock on an SM.  An eager
+// force evaluation with separate launches and so: 266 and 182 us at 1000
+// uniform particles, 351 and 285 at 4096 of a Plummer sphere.  At 6000 the
+// block takes as long as the launches (build 177 against 181 us), at 8192
+// longer (201 against 176).
 // The results are those of the separate launches, element for element.
 #define SM_T 1024
 #define SM_W (SM_T / NB_WARP)
-#define SM_I (NB_SMALL_N / SM_T)   // keys per thread at most
+#define SM_NEXT 12288   // nodes whose preorder successors fit in shared memory
 
 struct SmallSmem {
     uint64_t key[NB_SMALL_N];
     int32_t idx[NB_SMALL_N + 1];    // sorted order; then the scanned cell counts
-    uint32_t hist[SM_W][256];
-    uint32_t start[256];
+    int32_t next[SM_NEXT];
+    uint32_t depth[SM_W][32];
+    uint32_t start[32];
     int32_t wsum[SM_W];
     int8_t clev[NB_SMALL_N];
 };
@@ -1436,9 +1438,82 @@ __device__ __forceinline__ int32_t small_scan(int32_t v, int32_t *wsum, int32_t 
     return before + x - v;
 }
 
+// Order of the sort: by key, then by index (the stable order).
+__device__ __forceinline__ bool small_less(uint64_t ka, uint32_t va, uint64_t kb, uint32_t vb)
+{
+    return ka < kb || (ka == kb && va < vb);
+}
+
+// Bitonic sort of SM_T I (key, index) pairs, element tid I + r in register r
+// of thread tid: strides below I inside a thread, below 32 I by shuffles, the
+// others through shared memory.  (1000 keys: 6 us against 18 for eight passes
+// of the radix scatter inside the block, whose counts per warp and digit cost
+// the same for few keys as for many.)
+template <int I>
+__device__ __forceinline__ void small_sort(uint64_t (&k)[I], uint32_t (&v)[I], SmallSmem &S)
+{
+    const int tid = threadIdx.x;
+#pragma unroll 1
+    for (int size = 2; size <= SM_T * I; size <<= 1) {
+#pragma unroll 1
+        for (int stride = size >> 1; stride >= 32 * I; stride >>= 1) {
+            const int m = stride / I;
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < I; r++) {
+                S.key[r * SM_T + tid] = k[r];
+                S.idx[r * SM_T + tid] = (int32_t)v[r];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < I; r++) {
+                const uint64_t ko = S.key[r * SM_T + (tid ^ m)];
+                const uint32_t vo = (uint32_t)S.idx[r * SM_T + (tid ^ m)];
+                const bool up = ((tid * I + r) & size) == 0, low = (tid & m) == 0;
+                if (small_less(ko, vo, k[r], v[r]) == (up == low)) {
+                    k[r] = ko;
+                    v[r] = vo;
+                }
+            }
+        }
+#pragma unroll 1
+        for (int stride = min(size >> 1, 16 * I); stride >= I; stride >>= 1) {
+            const int m = stride / I;
+#pragma unroll
+            for (int r = 0; r < I; r++) {
+                const uint64_t ko = __shfl_xor_sync(0xffffffffu, k[r], m);
+                const uint32_t vo = __shfl_xor_sync(0xffffffffu, v[r], m);
+                const bool up = ((tid * I + r) & size) == 0, low = (tid & m) == 0;
+                if (small_less(ko, vo, k[r], v[r]) == (up == low)) {
+                    k[r] = ko;
+                    v[r] = vo;
+                }
+            }
+        }
+#pragma unroll
+        for (int stride = I / 2; stride >= 1; stride >>= 1)
+            if (stride <= (size >> 1))
+#pragma unroll
+                for (int r = 0; r < I; r++) {
+                    const int q = r ^ stride;
+                    if (q < r) continue;
+                    const bool up = ((tid * I + r) & size) == 0;
+                    if (small_less(k[q], v[q], k[r], v[r]) == up) {
+                        const uint64_t kt = k[r];
+                        const uint32_t vt = v[r];
+                        k[r] = k[q];
+                        v[r] = v[q];
+                        k[q] = kt;
+                        v[q] = vt;
+                    }
+                }
+    }
+}
+
 // Sort of (key, index), cells, their ends, parents and children, and the
-// level order.  Pointers written here are read here again: no read-only
-// loads (no const __restrict__) on them.
+// level order; I keys per thread.  Pointers written here are read here again:
+// no read-only loads (no const __restrict__) on them.
+template <int I>
 __global__ void __launch_bounds__(SM_T, 1)
 k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t *n_level,
                  int32_t *n_first, int32_t *n_count, int32_t *n_parent, int32_t *n_nchild,
@@ -1451,81 +1526,34 @@ k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t 
     const unsigned FULL = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int I = (n + SM_T - 1) / SM_T;   // keys per thread
-
-    // stable LSD radix sort, 8-bit digits: a warp holds I rounds of 32
-    // consecutive keys in registers, ranks them round by round (ballot match,
-    // running counts) and writes them back to shared memory in digit order
-    uint64_t k[SM_I];
-    uint32_t v[SM_I];
-    int e[SM_I];
+    uint64_t k[I];
+    uint32_t v[I];
 #pragma unroll
-    for (int r = 0; r < SM_I; r++) {
-        e[r] = r < I ? (w * I + r) * NB_WARP + lane : n;
-        k[r] = e[r] < n ? key[e[r]] : 0ull;
-        v[r] = (uint32_t)e[r];
+    for (int r = 0; r < I; r++) {   // (padding sorts to the end)
+        const int e = r * SM_T + tid;
+        k[r] = e < n ? key[e] : ~0ull;
+        v[r] = (uint32_t)e;
     }
-    for (int shift = 0; shift < 64; shift += 8) {
-        for (int i = tid; i < SM_W * 256; i += SM_T) (&S.hist[0][0])[i] = 0u;
-        __syncthreads();
-        uint32_t rnk[SM_I];
+    small_sort<I>(k, v, S);
+    __syncthreads();
 #pragma unroll
-        for (int r = 0; r < SM_I; r++) {
-            if (r >= I) break;
-            const bool ok = e[r] < n;
-            const int d = (int)((k[r] >> shift) & 255u);
-            const unsigned peers = nb_match_bits<8>((unsigned)d, ok);
-            const unsigned before = __popc(peers & lt);
-            const uint32_t pre = ok ? S.hist[w][d] : 0u;
-            __syncwarp();
-            if (ok && before == 0) S.hist[w][d] = pre + __popc(peers);
-            __syncwarp();
-            rnk[r] = pre + before;
+    for (int r = 0; r < I; r++) {
+        const int a = tid * I + r;
+        if (a < n) {
+            key[a] = k[r];
+            idx[a] = v[r];
         }
-        __syncthreads();
-        int32_t run = 0;
-        if (tid < 256)
-#pragma unroll 8
-            for (int ww = 0; ww < SM_W; ww++) {
-                const uint32_t c = S.hist[ww][tid];
-                S.hist[ww][tid] = (uint32_t)run;
-                run += (int32_t)c;
-            }
-        int32_t all;
-        const int32_t st = small_scan(run, S.wsum, &all);
-        if (tid < 256) S.start[tid] = (uint32_t)st;
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < SM_I; r++)
-            if (e[r] < n) {
-                const int d = (int)((k[r] >> shift) & 255u);
-                const uint32_t pos = S.start[d] + S.hist[w][d] + rnk[r];
-                if (!nb_in(pos < (uint32_t)n, cnt, err, SITE_SORT, pos)) continue;
-                S.key[pos] = k[r];
-                S.idx[pos] = (int32_t)v[r];
-            }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < SM_I; r++)
-            if (e[r] < n) {
-                k[r] = S.key[e[r]];
-                v[r] = (uint32_t)S.idx[e[r]];
-            }
+        S.key[a] = k[r];
     }
-#pragma unroll
-    for (int r = 0; r < SM_I; r++)
-        if (e[r] < n) {
-            key[e[r]] = k[r];
-            idx[e[r]] = v[r];
-        }
+    __syncthreads();
 
     // cells per particle, scanned (a thread's I consecutive particles)
-    int32_t cc[SM_I], mine = 0;
+    int32_t cc[I], mine = 0;
 #pragma unroll
-    for (int r = 0; r < SM_I; r++) {
+    for (int r = 0; r < I; r++) {
         const int a = tid * I + r;
         cc[r] = 0;
-        if (r < I && a < n) {
+        if (a < n) {
             const int ca = a + 1 < n ? common_levels(S.key[a], S.key[a + 1]) : -1;
             const int cp = a > 0 ? common_levels(S.key[a - 1], S.key[a]) : -1;
             S.clev[a] = (int8_t)ca;
@@ -1534,12 +1562,12 @@ k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t 
         mine += cc[r];
     }
     int32_t C;
-    int32_t at = small_scan(mine, S.wsum, &C);   // (its barriers: idx is read)
+    int32_t at = small_scan(mine, S.wsum, &C);
     int32_t *cst = S.idx;
 #pragma unroll
-    for (int r = 0; r < SM_I; r++) {
+    for (int r = 0; r < I; r++) {
         const int a = tid * I + r;
-        if (r < I && a < n) cst[a] = at;
+        if (a < n) cst[a] = at;
         at += cc[r];
     }
     if (tid == 0) {
@@ -1548,6 +1576,7 @@ k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t 
     }
     __syncthreads();
     const int32_t total = C + n;
+    const bool near = total <= SM_NEXT;   // successors in shared memory
 
     // nodes: leaves and cells by their first particle, and the cells' ends
     int deepest = -1;
@@ -1555,7 +1584,8 @@ k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t 
         deepest = max(deepest, cell_records(a, n, S.clev, cst, node_c, n_level, n_first, n_count,
                                             n_parent, n_nchild, n_depth, cnt, err));
         const int ca = S.clev[a], cp = a > 0 ? S.clev[a - 1] : -1;
-        const int32_t base = cst[a] + a;
+        const int32_t base = cst[a] + a, leaf = base + (ca > cp ? ca - cp : 0);
+        if (near) S.next[leaf] = leaf + 1;
         for (int lev = ca; lev > cp; lev--) {
             const int shift = 63 - 3 * lev;
             const uint64_t P = S.key[a] >> shift;
@@ -1572,17 +1602,19 @@ k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t 
                 else hi = mid;
             }
             const int32_t id = base + (lev - cp - 1);
-            node_c[id] = make_int4(cst[lo + 1] + lo + 1, 0, 0, 0);
+            const int32_t nx = cst[lo + 1] + lo + 1;
+            node_c[id] = make_int4(nx, 0, 0, 0);
             n_count[id] = lo - a + 1;
+            if (near) S.next[id] = nx;
         }
     }
     deepest = __reduce_max_sync(FULL, deepest);
     if (lane == 0 && deepest >= 0) atomicMax(&cnt[CNT_MAXLEVEL], (long long)deepest);
-    for (int i = tid; i < SM_W * 32; i += SM_T) (&S.hist[0][0])[i] = 0u;
+    (&S.depth[0][0])[tid] = 0u;
     __syncthreads();
 
     // parents and child counts; nodes per depth in each warp's run of nodes
-    uint32_t(*dh)[32] = reinterpret_cast<uint32_t(*)[32]>(&S.hist[0][0]);
+    uint32_t(*dh)[32] = S.depth;
     const int32_t per = ((total + SM_T - 1) / SM_T) * NB_WARP;   // nodes of a warp
     const int32_t u0 = w * per, u1 = min(u0 + per, total);
     for (int32_t ub = u0; ub < u1; ub += NB_WARP) {
@@ -1591,14 +1623,15 @@ k_topology_small(uint64_t *key, uint32_t *idx, int32_t n, int4 *node_c, int32_t 
         if (ok) {
             arrive[u] = 0;
             lcount[u] = 0;
-            const int4 cu = node_c[u];
-            if (!cu.w && nb_in(cu.x <= total, cnt, err, SITE_PARENTS, cu.x)) {
+            // (a leaf's successor is the node after it)
+            const int32_t un = near ? S.next[u] : node_c[u].x;
+            if (un > u + 1 && nb_in(un <= total, cnt, err, SITE_PARENTS, un)) {
                 int32_t ch = u + 1, nch = 0;
-                while (ch < cu.x) {
+                while (ch < un) {
                     n_parent[ch] = u;
                     nch++;
-                    const int32_t nx = node_c[ch].x;
-                    ch = nx > ch ? nx : cu.x;   // next always advances
+                    const int32_t nx = near ? S.next[ch] : node_c[ch].x;
+                    ch = nx > ch ? nx : un;   // next always advances
                 }
                 n_nchild[u] = nch;
             }
@@ -1743,18 +1776,28 @@ k_groups_small(const int32_t *__restrict__ n_count, const int32_t *__restrict__ 
     if (tid == 0) cnt[CNT_ITEMS] = done;
 }
 
-static void launch_topology_small(nb_ctx *c, int64_t n)
+template <int I>
+static void launch_topology_small_t(nb_ctx *c, int64_t n)
 {
     static bool done = false;
     if (!done) {
-        cudaFuncSetAttribute(k_topology_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_topology_small<I>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(SmallSmem));
         done = true;
     }
-    nb_launch(k_topology_small, 1, SM_T, sizeof(SmallSmem), nb_queue(c), c->keys, c->idx, (int)n,
-              c->node_c, c->n_level, c->n_first, c->n_count, c->n_parent, c->n_nchild, c->n_depth,
-              c->bfs2pid, c->pid2bfs, c->level_start, c->arrive, c->lcount, c->cnt, c->err);
+    nb_launch(k_topology_small<I>, 1, SM_T, sizeof(SmallSmem), nb_queue(c), c->keys, c->idx,
+              (int)n, c->node_c, c->n_level, c->n_first, c->n_count, c->n_parent, c->n_nchild,
+              c->n_depth, c->bfs2pid, c->pid2bfs, c->level_start, c->arrive, c->lcount, c->cnt,
+              c->err);
     nb_launched(c, "k_topology_small");
+}
+
+static void launch_topology_small(nb_ctx *c, int64_t n)
+{
+    static_assert(NB_SMALL_N == 4 * SM_T, "at most four keys per thread");
+    if (n <= SM_T) launch_topology_small_t<1>(c, n);
+    else if (n <= 2 * SM_T) launch_topology_small_t<2>(c, n);
+    else launch_topology_small_t<4>(c, n);
 }
 
 // Targets per force work item.  An item is one warp's work from start to end,

@@ -1,5 +1,6 @@
 """Sizes where the launches and the force work items change: one block builds
-the topology and the groups up to 8192 particles (1024 threads), items hold 8
+the topology and the groups up to 4096 particles (1024 threads, 1, 2 or 4 keys
+each), items hold 8
 targets up to 8192 particles, 16 up to 32,768, then 32.  Trees, groups and
 lists must equal the oracle's bit for bit on both sides of every line, forces
 meet the tolerances of the parity tests, and the fused and overlapped passes
@@ -21,7 +22,8 @@ if not torch.cuda.is_available():
 
 @pytest.mark.parametrize("order", ["morton", "hilbert"])
 @pytest.mark.parametrize("n,n_crit", [(1, 1), (2, 1), (33, 8), (1023, 32), (1024, 1), (1025, 64),
-                                      (5000, 8192), (8191, 17), (8192, 64), (8193, 64)])
+                                      (2048, 17), (2049, 64), (3000, 8192), (4095, 17), (4096, 64),
+                                      (4097, 64), (8193, 64)])
 def test_tree_groups_lists(oracle_lib, n, n_crit, order):
     ps = nbsynth.halo_mix(n, 60 + n, n_halos=5) if n > 100 else nbsynth.plummer(n, 60 + n)
     g = gpu_run(ps.pos, ps.mass, theta=0.7, n_crit=n_crit, eps=1e-3, key_order=order)
@@ -31,7 +33,7 @@ def test_tree_groups_lists(oracle_lib, n, n_crit, order):
         assert_lists_equal(g, T, 0.7, n_crit)
 
 
-@pytest.mark.parametrize("n", [4000, 8192])
+@pytest.mark.parametrize("n", [1000, 2000, 4096])
 def test_deep_chains_and_coincident_points(oracle_lib, n):
     """Pairs 1e-6 apart and coincident points: cells down to the last level,
     several nodes per particle."""
