@@ -17,15 +17,18 @@
 // run of sorted slots, and testing them all costs less than walking to their
 // leaves (runs of 4 and of 15: 2 and 4 % slower than 8 on that set).
 //
-// Candidates are gathered in shared memory and tested 64 at a time, two per
-// lane, against the members of the group (up to 64 of them, held in shared
+// The particles reached are gathered in shared memory; those farther than h
+// from the group's box are dropped, and the rest, the candidates, are tested
+// 64 at a time, two per lane, against the members of the group (up to 64 of them, held in shared
 // memory; a larger group is walked once per 64 members).  The test runs in
 // FP32 on group-relative coordinates and decides every pair whose distance
 // is not within rounding of h (band below); the FP64 definition is evaluated
 // only for pairs inside the band, so the result is the definition's.  On
 // GB300 the FP64 pipe gives about 1/64 of the FP32 lanes: with the FP64 test
 // on every pair, and the counts kept in global memory, a pass over 300,000
-// uniform points with 48 neighbours each took 7.2 ms; it takes 0.35 ms so (the fill pass 0.46 ms against 7.3).
+// uniform points with 48 neighbours each took 7.2 ms; it takes 0.30 ms (the
+// fill pass 0.39 against 7.3), and took 0.35 (0.46) without the test against
+// the box.
 // The first pass counts, an exclusive scan gives the offsets, the second
 // pass writes the caller indices, and each target's run is then sorted
 // ascending: runs of up to 256 in registers by a bitonic network, longer
@@ -40,8 +43,8 @@
 #define NG_RUN 8      // cells of at most this many particles are taken whole
 #define NG_MEM 64     // group members per work item
 #define NG_CHUNK 64   // candidates tested at a time (two per lane)
-// candidates kept over from one frontier chunk plus those one chunk can add
-#define NG_CAND (NG_CHUNK + NB_WARP * NG_RUN)
+// slots kept over from one frontier chunk plus those one chunk can add
+#define NG_RAW (NG_CHUNK + NB_WARP * NG_RUN)
 
 __device__ __forceinline__ double pair_d2(const double *a, const double *b)
 {
@@ -52,7 +55,8 @@ __device__ __forceinline__ double pair_d2(const double *a, const double *b)
 struct NeighWarp {
     int32_t qa[NG_SMEM], qb[NG_SMEM];
     float4 mem[NG_MEM];       // the item's members, group-relative
-    int32_t cand[NG_CAND];    // sorted slots of the candidates
+    int32_t raw[NG_RAW];      // sorted slots the walk reached
+    int32_t cand[2 * NG_CHUNK];   // those near the group's box: the candidates
 };
 
 // The band of FP32 squared distances that does not decide |d| <= h: at most
@@ -166,6 +170,30 @@ __device__ __forceinline__ void neigh_chunk(const NeighWarp &W, const int32_t *c
     }
 }
 
+// The slots raw[0 .. nr) (at most 64) that lie within reach of the group's
+// box, appended to the candidates; returns their new number.
+__device__ __forceinline__ int32_t neigh_near(NeighWarp &W, const int32_t *raw, int32_t nr,
+                                              int32_t nc, const float4 &blo, const float4 &bhi,
+                                              float reach, const float4 *__restrict__ p_hi,
+                                              int lane, unsigned lt)
+{
+    const unsigned FULL = 0xffffffffu;
+    int32_t s[2];
+    bool keep[2];
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        const int32_t e = q * NB_WARP + lane;
+        s[q] = raw[e < nr ? e : 0];
+        keep[q] = e < nr && !far_enough(p_hi[s[q]], reach, 0.0f, blo, bhi, 1.0f);
+    }
+    const unsigned m0 = __ballot_sync(FULL, keep[0]), m1 = __ballot_sync(FULL, keep[1]);
+    const int32_t n0 = __popc(m0);
+    if (keep[0]) W.cand[nc + __popc(m0 & lt)] = s[0];
+    if (keep[1]) W.cand[nc + n0 + __popc(m1 & lt)] = s[1];
+    __syncwarp();
+    return nc + n0 + __popc(m1);
+}
+
 // FILL false: count[perm[slot]] = neighbours; FILL true: write them at
 // off[i] ...  One warp per work item: the force items that start at a
 // multiple of 64 members give every group's runs of 64 members.
@@ -235,7 +263,12 @@ k_neigh(const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ items,
         int32_t *qin = qa, *qout = qb, *qin_s = W.qa, *qout_s = W.qb;
         if (lane == 0) qin_s[0] = sys_root ? sys_root[gsys] : 0;
         __syncwarp();
-        int32_t na = 1, nc = 0;
+        int32_t na = 1, nr = 0, nc = 0;
+        auto chunk = [&](int32_t from, int32_t m) {
+            neigh_chunk<FILL>(W, W.cand + from, m, f0, mt, bc, lo2, hi2, h2, p_hi, p_lo, x64, perm,
+                              idx, cap, lane, lt, cur0, cur1, bad);
+            __syncwarp();
+        };
         int depth_guard = 0;
         while (na > 0) {
             int32_t nb = 0;
@@ -268,7 +301,7 @@ k_neigh(const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ items,
                         }
                     }
                 }
-                // runs of candidates into the buffer
+                // runs of slots into the buffer
                 int32_t excl = 0;
 #pragma unroll
                 for (int q = 0; q < 4; q++)
@@ -276,13 +309,16 @@ k_neigh(const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ items,
                 const int32_t got = __reduce_add_sync(FULL, take);
 #pragma unroll
                 for (int k = 0; k < NG_RUN; k++)
-                    if (k < take) W.cand[nc + excl + k] = first + k;
-                nc += got;
+                    if (k < take) W.raw[nr + excl + k] = first + k;
+                nr += got;
                 __syncwarp();
-                while (nc >= NG_CHUNK) {
-                    nc -= NG_CHUNK;
-                    neigh_chunk<FILL>(W, W.cand + nc, NG_CHUNK, f0, mt, bc, lo2, hi2, h2, p_hi, p_lo,
-                                      x64, perm, idx, cap, lane, lt, cur0, cur1, bad);
+                while (nr >= NG_CHUNK) {
+                    nr -= NG_CHUNK;
+                    nc = neigh_near(W, W.raw + nr, NG_CHUNK, nc, blo, bhi, reach, p_hi, lane, lt);
+                    if (nc >= NG_CHUNK) {
+                        nc -= NG_CHUNK;
+                        chunk(nc, NG_CHUNK);
+                    }
                 }
                 __syncwarp();
                 // children of opened cells to the next level's queue
@@ -318,9 +354,12 @@ k_neigh(const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ items,
             na = nb;
             if (++depth_guard > NB_DEPTHS + 1) { bad |= NB_EF_WALK; break; }
         }
-        if (nc > 0)
-            neigh_chunk<FILL>(W, W.cand, nc, f0, mt, bc, lo2, hi2, h2, p_hi, p_lo, x64, perm, idx,
-                              cap, lane, lt, cur0, cur1, bad);
+        if (nr > 0) nc = neigh_near(W, W.raw, nr, nc, blo, bhi, reach, p_hi, lane, lt);
+        if (nc > NG_CHUNK) {
+            nc -= NG_CHUNK;
+            chunk(nc, NG_CHUNK);
+        }
+        if (nc > 0) chunk(0, nc);
         // every particle found itself once (distance 0)
         if (FILL) {   // each run must end where the next one starts
             if (t0 >= 0 && cur0 != off[t0 + 1]) bad |= NB_EF_BOUNDS;
