@@ -218,8 +218,9 @@ __device__ __forceinline__ void st_relaxed(uint32_t *p, uint32_t v)
 }
 
 // I keys per thread: a tile of RS_T * I keys (RS_I for the fixed-tile paths,
-// RS_I1 for the context's single-pass sort)
-template <bool ONESWEEP, int I = RS_I>
+// RS_I1 for the context's single-pass sort).  BYVAL: the digit is one of the
+// value's (the system packed above the particle index), not the key's.
+template <bool ONESWEEP, int I = RS_I, bool BYVAL = false>
 __global__ void __launch_bounds__(RS_T, 3)
 k_rs_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
              uint64_t *__restrict__ kout, uint32_t *__restrict__ vout,
@@ -251,16 +252,21 @@ k_rs_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
     const int wbase = w * (TILE / RS_WARPS);
     const unsigned lt = (1u << lane) - 1u;
     uint64_t key[I];
-    uint32_t rnk[I];
+    uint32_t rnk[I], val[I];
 #pragma unroll
     for (int r = 0; r < I; r++) {
         const int e = wbase + r * NB_WARP + lane;
-        key[r] = e < tn ? kin[tile0 + e] : 0ull;
+        key[r] = !BYVAL && e < tn ? kin[tile0 + e] : 0ull;
+        val[r] = BYVAL && e < tn ? vin[tile0 + e] : 0u;
     }
+    auto digit = [&](int r) -> int {
+        if constexpr (BYVAL) return (int)((val[r] >> shift) & 255u);
+        else return (int)((key[r] >> shift) & 255u);
+    };
 #pragma unroll
     for (int r = 0; r < I; r++) {
         const bool ok = wbase + r * NB_WARP + lane < tn;
-        const int d = ok ? (int)((key[r] >> shift) & 255u) : 256 + lane;
+        const int d = ok ? digit(r) : 256 + lane;
         const unsigned peers = nb_match_bits<8>((unsigned)d, ok);
         const unsigned before = __popc(peers & lt);
         const uint32_t pre = ok ? whist[w][d] : 0u;
@@ -343,18 +349,18 @@ k_rs_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
     for (int ww = 0; ww < RS_WARPS; ww++) wpre += ww < w ? wtot[ww] : 0u;
     lstart[t] = wpre + x - run;
     __syncthreads();
-    // values are loaded only now (they need no ranking): fewer registers
-    // held through the ranking rounds
-    uint32_t val[I];
+    // values (BYVAL: keys) are loaded only now, as they need no ranking: fewer
+    // registers held through the ranking rounds
 #pragma unroll
     for (int r = 0; r < I; r++) {
         const int e = wbase + r * NB_WARP + lane;
-        val[r] = e < tn ? vin[tile0 + e] : 0u;
+        if (BYVAL) key[r] = e < tn ? kin[tile0 + e] : 0ull;
+        else val[r] = e < tn ? vin[tile0 + e] : 0u;
     }
 #pragma unroll
     for (int r = 0; r < I; r++) {
         if (wbase + r * NB_WARP + lane < tn) {
-            const int d = (int)((key[r] >> shift) & 255u);
+            const int d = digit(r);
             const uint32_t lp = lstart[d] + whist[w][d] + rnk[r];
             if (lp < (uint32_t)tn) {
                 sk[lp] = key[r];
@@ -368,7 +374,7 @@ k_rs_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
 #pragma unroll 4
     for (int e = t; e < tn; e += RS_T) {
         const uint64_t k = sk[e];
-        const int d = (int)((k >> shift) & 255u);
+        const int d = BYVAL ? (int)((sv[e] >> shift) & 255u) : (int)((k >> shift) & 255u);
         const uint32_t pos = boff[d] + (uint32_t)e - lstart[d];
         if (pos >= n) {   // a self-check (recorded when a context is given)
             if (cnt) nb_bad(cnt, err, SITE_SORT, pos);
@@ -399,6 +405,8 @@ static void rs_setup()
                          RS_SMEM);
     cudaFuncSetAttribute(k_rs_scatter<true, RS_I1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          rs_smem(RS_I1));
+    cudaFuncSetAttribute(k_rs_scatter<true, RS_I1, true>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, rs_smem(RS_I1));
     done = true;
 }
 
@@ -464,6 +472,45 @@ void nb_radix_sort(nb_ctx *c, int64_t n)
         uint32_t *tv = va; va = vb; vb = tv;
     }
     // 8 passes: the result is back in c->keys / c->idx
+}
+
+// particles per digit of the system number (low byte, then high byte), from
+// the systems' offsets
+__global__ void __launch_bounds__(256)
+k_rs_sys_hist(const int64_t *__restrict__ off, int64_t nsys, uint32_t *__restrict__ hist)
+{
+    nb_grid_wait();
+    for (int64_t sy = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sy < nsys;
+         sy += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t size = (uint32_t)(off[sy + 1] - off[sy]);
+        atomicAdd(&hist[sy & 255], size);
+        atomicAdd(&hist[256 + ((sy >> 8) & 255)], size);
+    }
+}
+
+// Sort the key-sorted (c->keys, c->idx) stably by the system number held in
+// the values from bit `bits` on (nsys <= 65536): one or two more single-pass
+// digits.  False if the status words have no room (the caller sorts by other
+// means).  Result in c->keys / c->idx.
+bool nb_radix_sort_systems(nb_ctx *c, const int64_t *off, int64_t nsys, int64_t n, int bits)
+{
+    const int nb = (int)((n + (int64_t)RS_T * RS_I1 - 1) / ((int64_t)RS_T * RS_I1));
+    const int64_t words = (int64_t)nb * 256 * 2 + 2 * 256 + 2;
+    if (n >= (int64_t)RS_VAL || words > c->rs_status_len) return false;
+    rs_setup();
+    uint32_t *hist = c->rs_status + (int64_t)nb * 256 * 2, *ctr = hist + 2 * 256;
+    cudaMemsetAsync(c->rs_status, 0, sizeof(uint32_t) * words, c->stream);
+    nb_launch(k_rs_sys_hist, nb_grid(nsys, 256, c->num_sms), 256, 0, nb_queue(c), off, nsys, hist);
+    nb_launched(c, "k_rs_sys_hist");
+    for (int pass = 0; pass < (nsys > 256 ? 2 : 1); pass++) {
+        nb_launch(k_rs_scatter<true, RS_I1, true>, nb, RS_T, rs_smem(RS_I1), nb_queue(c), c->keys,
+                  c->idx, c->keys_alt, c->idx_alt, nullptr, n, bits + 8 * pass, nb, c->cnt, c->err,
+                  c->rs_status + (int64_t)pass * nb * 256, hist + 256 * pass, ctr + pass);
+        nb_launched(c, "k_rs_scatter");
+        uint64_t *tk = c->keys; c->keys = c->keys_alt; c->keys_alt = tk;
+        uint32_t *tv = c->idx; c->idx = c->idx_alt; c->idx_alt = tv;
+    }
+    return true;
 }
 
 // ------------------------------------------------------- explicit buffers

@@ -257,7 +257,7 @@ __device__ __forceinline__ void hilbert_point(uint64_t key, uint32_t q[3])
 __global__ void __launch_bounds__(256)
 k_keys(const double *__restrict__ pos, int64_t n, const double *__restrict__ roots,
        const int32_t *__restrict__ sys_of, uint64_t *__restrict__ key, uint32_t *__restrict__ idx,
-       int hilbert)
+       int hilbert, int pack)
 {
     nb_grid_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -269,7 +269,8 @@ k_keys(const double *__restrict__ pos, int64_t n, const double *__restrict__ roo
     const uint32_t qz = grid_coord(pos[3 * i + 2], root[6], sc);
     key[i] = hilbert ? hilbert_key(qx, qy, qz)
                      : (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
-    idx[i] = (uint32_t)i;
+    // pack > 0: the particle's system above `pack` bits of its index
+    idx[i] = (uint32_t)i | (pack ? (uint32_t)sys_of[i] << pack : 0u);
 }
 
 // sorted slot s: gather the caller's particle idx[s]; split FP64 positions
@@ -966,7 +967,7 @@ void nb_launch_build(nb_ctx *c, const double *pos, const float *mass, int64_t n)
               c->cnt, c->root);
     nb_launched(c, "k_bbox_root");
     nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(c), pos, n, c->root, nullptr, c->keys,
-              c->idx, c->key_order);
+              c->idx, c->key_order, 0);
     nb_launched(c, "k_keys");
     if (nb_small_system(c)) launch_topology_small(c, n);
     else nb_radix_sort(c, n);
@@ -1100,21 +1101,30 @@ k_sys_roots(const int32_t *__restrict__ level_start, const int32_t *__restrict__
         sys_root[sys_sorted[n_first[bfs2pid[b]]]] = b;
 }
 
-void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, int64_t n,
-                             const int64_t *off, int64_t nsys)
+// the values' packed systems and indices apart (a system number beyond the
+// batch can only come from offsets that the offset check has reported)
+__global__ void __launch_bounds__(256)
+k_sys_unpack(uint32_t *__restrict__ idx, int64_t n, int bits, int64_t nsys,
+             int32_t *__restrict__ sys_sorted)
+{
+    nb_grid_wait();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t v = idx[i];
+    sys_sorted[i] = (int32_t)min((int64_t)(v >> bits), nsys - 1);
+    idx[i] = v & ((1u << bits) - 1u);
+}
+
+// the key-sorted particles stably by system: a sort of the gathered system
+// numbers, applied to keys and indices
+static void sort_by_system(nb_ctx *c, int64_t n, int packed)
 {
     cudaStream_t s = c->stream;
-    cudaMemsetAsync(c->cnt, 0, sizeof(long long) * CNT_PP_CUM, s);
-    const int gs = (int)(nsys < 65535 ? nsys : 65535);
-    nb_launch(k_sys_of, gs, 256, 0, nb_queue(c), off, nsys, n, c->sys_of, c->err);
-    nb_launched(c, "k_sys_of");
-    nb_launch(k_roots_sys, gs, RS_SYS_T, 0, nb_queue(c), pos, off, nsys, n, c->root, c->err);
-    nb_launched(c, "k_roots_sys");
-    nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(c), pos, n, c->root, c->sys_of, c->keys,
-              c->idx, c->key_order);
-    nb_launched(c, "k_keys");
-    nb_radix_sort(c, n);
-    // stable by system on top of the Morton order: (system, key) order
+    if (packed) {
+        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, packed,
+                  c->nsys, c->sys_sorted);
+        nb_launched(c, "k_sys_unpack");
+    }
     nb_launch(k_sys_key, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, c->sys_of, n, c->skey,
               c->sval);
     nb_launched(c, "k_sys_key");
@@ -1126,6 +1136,36 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
     nb_launched(c, "k_sys_apply");
     uint64_t *tk = c->keys; c->keys = c->keys_alt; c->keys_alt = tk;
     uint32_t *ti = c->idx; c->idx = c->idx_alt; c->idx_alt = ti;
+}
+
+void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, int64_t n,
+                             const int64_t *off, int64_t nsys)
+{
+    cudaStream_t s = c->stream;
+    cudaMemsetAsync(c->cnt, 0, sizeof(long long) * CNT_PP_CUM, s);
+    const int gs = (int)(nsys < 65535 ? nsys : 65535);
+    nb_launch(k_sys_of, gs, 256, 0, nb_queue(c), off, nsys, n, c->sys_of, c->err);
+    nb_launched(c, "k_sys_of");
+    nb_launch(k_roots_sys, gs, RS_SYS_T, 0, nb_queue(c), pos, off, nsys, n, c->root, c->err);
+    nb_launched(c, "k_roots_sys");
+    // the system rides in the high bits of the sorted values where both fit
+    // 32 bits, and one or two more digits sort by it; else a second sort of
+    // the gathered system numbers
+    int bits = 1, sbits = 1;
+    while ((n - 1) >> bits) bits++;
+    while ((nsys - 1) >> sbits) sbits++;
+    const bool pack = bits + sbits <= 32 && nsys <= 65536;
+    nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(c), pos, n, c->root, c->sys_of, c->keys,
+              c->idx, c->key_order, pack ? bits : 0);
+    nb_launched(c, "k_keys");
+    nb_radix_sort(c, n);
+    if (pack && nb_radix_sort_systems(c, off, nsys, n, bits)) {
+        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, bits,
+                  nsys, c->sys_sorted);
+        nb_launched(c, "k_sys_unpack");
+    } else {
+        sort_by_system(c, n, pack ? bits : 0);
+    }
     build_tail(c, pos, mass, n, c->sys_sorted);
     nb_launch(k_sys_roots, nb_grid(nsys, 256, c->num_sms * 4), 256, 0, nb_queue(c), c->level_start,
               c->bfs2pid, c->n_first, c->sys_sorted, c->sys_root);
@@ -1857,6 +1897,6 @@ void nb_launch_keys_raw(const double *pos, int64_t n, double *part, int nblk, do
     nb_launch(k_bbox, nblk, 256, 0, nb_queue(s, n), pos, n, part, err);
     nb_launch(k_root, 1, 256, 0, nb_queue(s, n), part, nblk, root);
     nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(s, n), pos, n, root, nullptr, keys, idx,
-              0);
+              0, 0);
 }
 

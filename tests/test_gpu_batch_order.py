@@ -1,0 +1,51 @@
+"""The (system, key) order of a batch where the system number rides in the
+sorted values: one digit up to 256 systems, two beyond, odd sizes, and equal
+keys (coincident particles keep the caller's order).  Every system's slots
+must be the stable key order of its own rows, with the keys that system's
+tree gets when it is built alone.
+"""
+import numpy as np
+import pytest
+
+import nbsynth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+
+@pytest.mark.parametrize("nsys,lo,hi", [(2, 1, 5000), (255, 1, 60), (256, 3, 40), (257, 1, 50),
+                                        (700, 1, 30)])
+def test_order_is_stable_by_system_and_key(nsys, lo, hi):
+    import paper_0909_0541_gb300 as nb
+    rng = np.random.default_rng(nsys)
+    size = rng.integers(lo, hi + 1, nsys)
+    off = np.concatenate([[0], np.cumsum(size)]).astype(np.int64)
+    n = int(off[-1])
+    pos = nbsynth.uniform_cube(n, 17 + nsys).pos * rng.uniform(0.1, 10.0)
+    for s in range(0, nsys, 3):            # coincident particles in some systems
+        if size[s] > 3:
+            pos[off[s] + 1:off[s] + 3] = pos[off[s]]
+    dev = torch.device("cuda")
+    x = torch.from_numpy(pos).to(dev)
+    m = torch.full((n,), 1.0 / n, dtype=torch.float32, device=dev)
+    ctx = nb.NBody(n, max_systems=nsys)
+    ctx.build_tree_batched(x, m, torch.from_numpy(off).to(dev))
+    t = ctx.copy_tree()
+    keys, perm = t["keys"], t["perm"]
+    assert np.array_equal(np.sort(perm), np.arange(n))
+    for s in range(nsys):
+        a, b = off[s], off[s + 1]
+        p, k = perm[a:b], keys[a:b]
+        assert p.min() >= a and p.max() < b, s
+        assert np.all((k[1:] > k[:-1]) | ((k[1:] == k[:-1]) & (p[1:] > p[:-1]))), s
+    for s in (0, nsys // 2, nsys - 1):
+        a, b = off[s], off[s + 1]
+        one = nb.NBody(int(b - a))
+        one.build_tree(x[a:b].contiguous(), m[a:b].contiguous())
+        o = one.copy_tree()
+        assert np.array_equal(o["keys"], keys[a:b]) and np.array_equal(o["perm"] + a, perm[a:b])
+        one.close()
+    ctx.close()
