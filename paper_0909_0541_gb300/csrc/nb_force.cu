@@ -365,10 +365,14 @@ static void launch_force_t(nb_ctx *c, float eps2, float *acc, float *pot)
                                                       k_force<MODE, GUARD, TILE, BT, QUAD>, BT, 0);
         if (blocks < 1) blocks = 1;
     }
-    nb_launch(k_force<MODE, GUARD, TILE, BT, QUAD>, c->num_sms * blocks, BT, 0, nb_queue(c),
-              c->items, nb_small_system(c) ? nullptr : c->item_order, c->gfirst, c->gcount,
-              c->glen, c->gbox, c->p_hi, c->p_lo, c->perm, c->list_xm, c->list_q, c->list_cap,
-              c->list_alloc, c->n, c->cnt, eps2, acc, pot, c->err, c->max_items);
+    // (a group has full items and at most two smaller ones)
+    const int64_t items = 2 * c->n / nb_item_block(c) + 2 * (16 * (c->n / c->n_crit_cur) + 64);
+    const int grid = nb_queue_blocks(items < c->max_items ? items : c->max_items, BT / NB_WARP,
+                                     c->num_sms * blocks);
+    nb_launch(k_force<MODE, GUARD, TILE, BT, QUAD>, grid, BT, 0, nb_queue(c), c->items,
+              nb_small_system(c) ? nullptr : c->item_order, c->gfirst, c->gcount, c->glen, c->gbox,
+              c->p_hi, c->p_lo, c->perm, c->list_xm, c->list_q, c->list_cap, c->list_alloc, c->n,
+              c->cnt, eps2, acc, pot, c->err, c->max_items);
     nb_launched(c, QUAD ? "k_force (quadrupole)" : "k_force");
 }
 

@@ -963,8 +963,8 @@ void nb_launch_build(nb_ctx *c, const double *pos, const float *mass, int64_t n)
 {
     cudaStream_t s = c->stream;
     cudaMemsetAsync(c->cnt, 0, sizeof(long long) * CNT_PP_CUM, s);
-    nb_launch(k_bbox_root, c->bbox_blocks, 256, 0, nb_queue(c), pos, n, c->bbox_part, c->err,
-              c->cnt, c->root);
+    nb_launch(k_bbox_root, nb_grid(n, 512, c->bbox_blocks), 256, 0, nb_queue(c), pos, n,
+              c->bbox_part, c->err, c->cnt, c->root);
     nb_launched(c, "k_bbox_root");
     nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(c), pos, n, c->root, nullptr, c->keys,
               c->idx, c->key_order, 0);
@@ -1121,8 +1121,8 @@ static void sort_by_system(nb_ctx *c, int64_t n, int packed)
 {
     cudaStream_t s = c->stream;
     if (packed) {
-        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, packed,
-                  c->nsys, c->sys_sorted);
+        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, packed, c->nsys,
+                  c->sys_sorted);
         nb_launched(c, "k_sys_unpack");
     }
     nb_launch(k_sys_key, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, c->sys_of, n, c->skey,
@@ -1160,8 +1160,8 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
     nb_launched(c, "k_keys");
     nb_radix_sort(c, n);
     if (pack && nb_radix_sort_systems(c, off, nsys, n, bits)) {
-        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, bits,
-                  nsys, c->sys_sorted);
+        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, bits, nsys,
+                  c->sys_sorted);
         nb_launched(c, "k_sys_unpack");
     } else {
         sort_by_system(c, n, pack ? bits : 0);
@@ -1230,14 +1230,18 @@ static void build_tail(nb_ctx *c, const double *pos, const float *mass, int64_t 
         if (mblocks < 1) mblocks = 1;
         if (qblocks < 1) qblocks = 1;
     }
+    // chunks of 32 cells: at most 11 cells per particle (on average well below
+    // one), and a partial chunk per bucket
+    const int mwarps = 256 / NB_WARP;
+    const int64_t chunks = n / 16 + NB_CBKT;
     if (c->quad && c->b_q)
-        nb_launch(k_moments<true>, c->num_sms * qblocks, 256, 0, nb_queue(c), c->clist,
-                  c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass, c->b_mx, c->b_com, c->b_q,
-                  c->arrive, c->cnt, c->err);
+        nb_launch(k_moments<true>, nb_queue_blocks(chunks, mwarps, c->num_sms * qblocks), 256, 0,
+                  nb_queue(c), c->clist, c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass,
+                  c->b_mx, c->b_com, c->b_q, c->arrive, c->cnt, c->err);
     else
-        nb_launch(k_moments<false>, c->num_sms * mblocks, 256, 0, nb_queue(c), c->clist,
-                  c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass, c->b_mx, c->b_com, nullptr,
-                  c->arrive, c->cnt, c->err);
+        nb_launch(k_moments<false>, nb_queue_blocks(chunks, mwarps, c->num_sms * mblocks), 256, 0,
+                  nb_queue(c), c->clist, c->clist_len, c->wrec, c->b_up, c->lcount, c->b_mass,
+                  c->b_mx, c->b_com, nullptr, c->arrive, c->cnt, c->err);
     nb_launched(c, "k_moments");
 }
 
@@ -1896,7 +1900,7 @@ void nb_launch_keys_raw(const double *pos, int64_t n, double *part, int nblk, do
 {
     nb_launch(k_bbox, nblk, 256, 0, nb_queue(s, n), pos, n, part, err);
     nb_launch(k_root, 1, 256, 0, nb_queue(s, n), part, nblk, root);
-    nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(s, n), pos, n, root, nullptr, keys, idx,
-              0, 0);
+    nb_launch(k_keys, nb_grid(n, 256), 256, 0, nb_queue(s, n), pos, n, root, nullptr, keys, idx, 0,
+              0);
 }
 

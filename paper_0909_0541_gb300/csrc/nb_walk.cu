@@ -147,12 +147,21 @@ int nb_walk_warps(nb_ctx *c)
     return c->num_sms * blocks * WALK_WARPS;
 }
 
+// blocks of one walk launch: a group has at most n_crit members and seldom
+// fewer than a sixteenth of that, so up to 16 n / n_crit groups get a warp each
+static int walk_blocks(nb_ctx *c)
+{
+    const int64_t crit = c->n_crit_cur > 1 ? c->n_crit_cur : 1;
+    const int64_t groups = 16 * (c->n / crit) + 64;
+    return nb_queue_blocks(groups < c->n ? groups : c->n, WALK_WARPS, c->walk_warps / WALK_WARPS);
+}
+
 void nb_launch_walk(nb_ctx *c)
 {
     cudaMemsetAsync(&c->cnt[CNT_LIST_TOT], 0, sizeof(long long) * 5, c->stream);
     static_assert(CNT_LIST_TOT + 4 == CNT_WALK_Q, "counter layout");
     cudaMemsetAsync(&c->cnt[CNT_QMAX], 0, sizeof(long long), c->stream);
-    const int blocks = c->walk_warps / WALK_WARPS;
+    const int blocks = walk_blocks(c);
     if (c->quad && c->b_q && c->list_q)
         nb_launch(k_walk<false, true>, blocks, WALK_T, 0, nb_queue(c), c->wrec, c->pid2bfs,
                   c->gnode, c->gcount, c->gbox, c->cnt, c->glen, c->gcells, c->list_id, c->list_xm,
