@@ -17,6 +17,8 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "nb_internal.cuh"
 
 #define MH 64
@@ -394,8 +396,10 @@ extern "C" int nb_theta_labels(const float *err_dev, const float *cost_dev,
 // A step is a chain of ten small dependent products and reductions, bound by
 // their latency, not by arithmetic (256 samples: 14 MFLOP).  As four launches
 // a step over device memory it took 94 us, most of it in weight and bias sums
-// that walked the batch in 11 blocks; it takes 10.2 us so (256 samples, a
-// cluster of 16 blocks).
+// that walked the batch in 11 blocks; it takes 9.8 us so (256 samples, a
+// cluster of 16 blocks; 10.2 before the bias sums took their tiles in two
+// alternating register sets and the next tile was put down between the two
+// halves of the step's last barrier).
 //
 // Phase A: a block takes one 16-sample tile (tile k of a round goes to block
 // k) forward and back.  Its 8 warps split a layer's 64 outputs, 8 columns
@@ -658,10 +662,23 @@ k_mlp_train(float *__restrict__ P, float *__restrict__ am, float *__restrict__ a
     int64_t i1 = next_sample();
     fetch(i1);
     i1 = next_sample();
+    // the tile's input rows and labels into shared memory; the next one's are
+    // fetched
+    auto put_input = [&](bool has_tile) {
+        if (has_tile) {
+            S.a0[row * MT_LD0 + col] = __float2bfloat16_rn(
+                ok1 && col < MNIN ? __fdiv_rn(__fsub_rn(x1, S.mu[col]), S.sg[col]) : 0.f);
+            if (col == 0) S.y[row] = y1;
+        }
+        fetch(i1);
+        i1 = next_sample();
+    };
     // the running loss of the current epoch (one lane of block 0)
     int64_t le = step0 / steps_per_epoch, lk = step0 - le * steps_per_epoch;
     float lrun = 0.f;
     if (rank == 0 && w == 6 && loss) lrun = loss[TRAIN ? le : 0];
+    __syncthreads();   // mu and sigma
+    put_input(rank < ntiles);
     cl.sync();
 
     for (int s = 0; s < nsteps; s++) {
@@ -673,14 +690,7 @@ k_mlp_train(float *__restrict__ P, float *__restrict__ am, float *__restrict__ a
         for (int64_t j = 0; j < rounds; j++) {
             const int64_t base = j * CL;                 // first tile of the round
             const int nk = ntiles - base < CL ? (int)(ntiles - base) : CL;
-            if (rank < nk) {
-                // ---- phase A: this block's tile
-                S.a0[row * MT_LD0 + col] = __float2bfloat16_rn(
-                    ok1 && col < MNIN ? __fdiv_rn(__fsub_rn(x1, S.mu[col]), S.sg[col]) : 0.f);
-                if (col == 0) S.y[row] = y1;
-            }
-            fetch(i1);
-            i1 = next_sample();
+            if (j > 0) put_input(rank < nk);
             __syncthreads();
             if (rank < nk) {
                 const int c0 = w * 8 + 2 * t;
@@ -830,25 +840,32 @@ k_mlp_train(float *__restrict__ P, float *__restrict__ am, float *__restrict__ a
                 } else if (w == 5) {
                     const bool prod = (vr >> 2) == 3;   // w4: dz h3; biases: dZ
                     const int c = lane & 15;
-                    // the column's rows in order, one tile's loads ahead of
-                    // the additions
-                    float sum = acc[v][0], x[16], y[16];
-                    auto load = [&](int k, float (&to)[16]) {
+                    // the column's rows in order; two tiles' loads in turn, so
+                    // that one is in flight while the other is added
+                    float sum = acc[v][0];
+                    auto chain = [&](auto product) {
+                        float x[2][16];
+                        auto load = [&](int k, float (&to)[16]) {
 #pragma unroll
-                        for (int r = 0; r < 16; r++) {
-                            to[r] = S.rf[v * CL + k][r * 16 + c];
-                            if (prod) to[r] = __fmul_rn(S.rdz[k][r], to[r]);
+                            for (int r = 0; r < 16; r++) to[r] = S.rf[v * CL + k][r * 16 + c];
+                            if constexpr (decltype(product)::value)
+#pragma unroll
+                                for (int r = 0; r < 16; r++) to[r] = __fmul_rn(S.rdz[k][r], to[r]);
+                        };
+                        auto add = [&](const float (&from)[16]) {
+#pragma unroll
+                            for (int r = 0; r < 16; r++) sum = __fadd_rn(sum, from[r]);
+                        };
+                        load(0, x[0]);
+                        for (int k = 0; k < nk; k += 2) {
+                            if (k + 1 < nk) load(k + 1, x[1]);
+                            add(x[0]);
+                            if (k + 2 < nk) load(k + 2, x[0]);
+                            if (k + 1 < nk) add(x[1]);
                         }
                     };
-                    load(0, x);
-                    for (int k = 0; k < nk; k++) {
-                        if (k + 1 < nk) load(k + 1, y);
-#pragma unroll
-                        for (int r = 0; r < 16; r++) {
-                            sum = __fadd_rn(sum, x[r]);
-                            x[r] = y[r];
-                        }
-                    }
+                    if (prod) chain(std::true_type{});
+                    else chain(std::false_type{});
                     acc[v][0] = sum;
                 } else if (w == 6 && rank == 0 && v == 0) {
                     for (int r = lane; r < nk * 16; r += 32) {
@@ -897,7 +914,11 @@ k_mlp_train(float *__restrict__ P, float *__restrict__ am, float *__restrict__ a
                     *to = p0;
             }
         }
-        cl.sync();
+        // the next step's first tile is put down while the blocks meet (the
+        // local tile was read before the last barrier)
+        cl.barrier_arrive();
+        if (s + 1 < nsteps) put_input(rank < ntiles);
+        cl.barrier_wait();
         if (TRAIN) {   // the new parameters
             for (int q = tid; q < (P_W4 + MH) / 4; q += MT_T)
                 fetch16(S.P + smem_place(4 * q), X.P + 4 * q);
