@@ -19,9 +19,10 @@
 //
 // The particles reached are gathered in shared memory; those farther than h
 // from the group's box are dropped, and the rest, the candidates, are tested
-// 64 at a time, two per lane, against the members of the group (up to 64 of them, held in shared
-// memory; a larger group is walked once per 64 members).  The test runs in
-// FP32 on group-relative coordinates and decides every pair whose distance
+// 64 at a time, two per lane, against the members of the group (up to 64 of
+// them, held in shared memory; a larger group is walked once per 64 members).
+// The test runs in FP32 on group-relative coordinates and decides every pair
+// whose distance
 // is not within rounding of h (band below); the FP64 definition is evaluated
 // only for pairs inside the band, so the result is the definition's.  On
 // GB300 the FP64 pipe gives about 1/64 of the FP32 lanes: with the FP64 test
