@@ -393,7 +393,7 @@ int nb_create(nb_ctx **out, const nb_config *cfg)
     c->sync_checks = cfg->sync_checks;
     if (cudaSetDevice(c->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) !=
-            cudaSuccess) {
+            cudaSuccess || nb_tree_setup()) {
         cudaGetLastError();
         delete c;
         return NB_ERR_CUDA;

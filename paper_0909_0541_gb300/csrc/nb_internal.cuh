@@ -286,6 +286,7 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
                              const int64_t *offsets, int64_t nsys);
 void nb_launch_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g);
 int nb_item_block(const nb_ctx *c);
+int nb_tree_setup();
 
 // nb_walk.cu
 int nb_walk_warps(nb_ctx *c);

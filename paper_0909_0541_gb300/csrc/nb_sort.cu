@@ -391,23 +391,20 @@ k_rs_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
 // fuller than 701 larger ones).  Any tile size gives the same sort.
 #define RS_I1 12
 
-// the staging buffer is dynamic shared memory above the 48 KB default
+// the staging buffer of a tile (dynamic shared memory)
 static constexpr int rs_smem(int I)
 {
     return RS_T * I * (int)(sizeof(uint64_t) + sizeof(uint32_t));
 }
+static_assert(rs_smem(RS_I1) + (RS_WARPS + 3) * 1024 <= 48 * 1024, "needs a raised limit");
 
+// The fixed tile's buffer and the kernel's static arrays are above 48 KB, the
+// single-pass tile's (36 + 10 KB) are not.  The limit belongs to the current
+// device: it is raised before every use (a host call, no work on the stream).
 static void rs_setup()
 {
-    static bool done = false;
-    if (done) return;
     cudaFuncSetAttribute(k_rs_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          RS_SMEM);
-    cudaFuncSetAttribute(k_rs_scatter<true, RS_I1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         rs_smem(RS_I1));
-    cudaFuncSetAttribute(k_rs_scatter<true, RS_I1, true>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, rs_smem(RS_I1));
-    done = true;
 }
 
 // all eight 8-bit digit histograms in one read of the keys: shared-memory
@@ -436,7 +433,6 @@ void nb_radix_sort(nb_ctx *c, int64_t n)
 {
     if (n <= 1) return;
     const int nb16 = (int)((n + RS_TILE - 1) / RS_TILE);
-    rs_setup();
     uint64_t *ka = c->keys, *kb = c->keys_alt;
     uint32_t *va = c->idx, *vb = c->idx_alt;
     const int nb = (int)((n + (int64_t)RS_T * RS_I1 - 1) / ((int64_t)RS_T * RS_I1));
@@ -459,6 +455,7 @@ void nb_radix_sort(nb_ctx *c, int64_t n)
         }
         return;   // 8 passes: the result is back in c->keys / c->idx
     }
+    rs_setup();
     for (int pass = 0; pass < 8; pass++) {
         const int shift = 8 * pass;
         nb_launch(k_rs_hist, nb16, RS_T, 0, nb_queue(c), ka, n, shift, c->sort_hist, nb16);
@@ -497,7 +494,6 @@ bool nb_radix_sort_systems(nb_ctx *c, const int64_t *off, int64_t nsys, int64_t 
     const int nb = (int)((n + (int64_t)RS_T * RS_I1 - 1) / ((int64_t)RS_T * RS_I1));
     const int64_t words = (int64_t)nb * 256 * 2 + 2 * 256 + 2;
     if (n >= (int64_t)RS_VAL || words > c->rs_status_len) return false;
-    rs_setup();
     uint32_t *hist = c->rs_status + (int64_t)nb * 256 * 2, *ctr = hist + 2 * 256;
     cudaMemsetAsync(c->rs_status, 0, sizeof(uint32_t) * words, c->stream);
     nb_launch(k_rs_sys_hist, nb_grid(nsys, 256, c->num_sms), 256, 0, nb_queue(c), off, nsys, hist);

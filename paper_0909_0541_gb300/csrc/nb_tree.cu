@@ -1820,15 +1820,20 @@ k_groups_small(const int32_t *__restrict__ n_count, const int32_t *__restrict__ 
     if (tid == 0) cnt[CNT_ITEMS] = done;
 }
 
+// The block's shared memory is above the 48 KB default.  The limit belongs to
+// the device, so every context raises it for its own (the current one).
+int nb_tree_setup()
+{
+    const cudaFuncAttribute lim = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const int bytes = (int)sizeof(SmallSmem);
+    return cudaFuncSetAttribute(k_topology_small<1>, lim, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_topology_small<2>, lim, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_topology_small<4>, lim, bytes) == cudaSuccess ? 0 : -1;
+}
+
 template <int I>
 static void launch_topology_small_t(nb_ctx *c, int64_t n)
 {
-    static bool done = false;
-    if (!done) {
-        cudaFuncSetAttribute(k_topology_small<I>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(SmallSmem));
-        done = true;
-    }
     nb_launch(k_topology_small<I>, 1, SM_T, sizeof(SmallSmem), nb_queue(c), c->keys, c->idx,
               (int)n, c->node_c, c->n_level, c->n_first, c->n_count, c->n_parent, c->n_nchild,
               c->n_depth, c->bfs2pid, c->pid2bfs, c->level_start, c->arrive, c->lcount, c->cnt,
