@@ -75,8 +75,8 @@ typedef struct nb_stats {
     int64_t n_pc;          /* particle-cell interactions                     */
     int32_t max_level;     /* deepest cell level                             */
     int32_t reserved;
-    int64_t n_pp_total;    /* n_pp summed over every walk of this context    */
-    int64_t n_pc_total;    /* n_pc summed over every walk of this context    */
+    int64_t n_pp_total;    /* n_pp summed over every walk of this context,   */
+    int64_t n_pc_total;    /* n_pc too (without walks repeated with more room) */
 } nb_stats;
 
 /* phases timed by nb_set_timing */

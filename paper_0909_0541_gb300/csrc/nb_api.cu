@@ -298,6 +298,17 @@ static int read_counters(nb_ctx *c)
     return NB_OK;
 }
 
+// take a walk that is to be repeated (its counts in cnt_host) out of the totals
+static int uncount(nb_ctx *c)
+{
+    static_assert(CNT_PC_CUM == CNT_PP_CUM + 1, "counter layout");
+    c->cnt_host[CNT_PP_CUM] -= c->cnt_host[CNT_PP];
+    c->cnt_host[CNT_PC_CUM] -= c->cnt_host[CNT_PC];
+    CK(cudaMemcpyAsync(&c->cnt[CNT_PP_CUM], &c->cnt_host[CNT_PP_CUM], 2 * sizeof(long long),
+                       cudaMemcpyHostToDevice, c->stream));
+    return NB_OK;
+}
+
 int nb_read_err(nb_ctx *c, unsigned *bits) { return sync_read_bits(c, bits); }
 int nb_err_code(unsigned bits) { return err_code(bits); }
 
@@ -536,64 +547,52 @@ static int walk_groups(nb_ctx *c, float theta, int n_crit, const float *theta_g,
     if (formed) nb_launch_group_theta(c, theta_g);
     else nb_launch_groups(c, theta, n_crit, theta_g);
     c->has_groups = 1;
-    if (c->sync_checks && c->list_alloc > 0 && c->list_cap > 0 && c->wq &&
-        !(c->quad && !c->list_q)) {
-        // storage from an earlier walk: walk at once, without waiting for the
-        // number of groups (the walk stays inside the storage and reports
-        // what does not fit; the loop below then sizes it and walks again)
-        nb_launch_walk(c);
-        if (cudaGetLastError() != cudaSuccess) return NB_ERR_CUDA;
-        unsigned bits = 0;
-        int rc = sync_read_all(c, &bits);
-        if (rc) return rc;
-        c->groups_host = c->cnt_host[CNT_GROUPS];
-        rc = err_code(bits);
-        if (rc != NB_ERR_CAPACITY) {
-            phase_end(c, tk, NB_PHASE_WALK);
-            if (rc) return rc;
-            c->has_lists = 1;
-            c->lists_quad = c->quad;
-            return NB_OK;
-        }
-    }
     if (c->sync_checks) {
-        int rc = read_counters(c);
+        // With storage from an earlier walk the first walk starts without
+        // waiting for the number of groups (it stays inside the storage and
+        // reports what does not fit).  With none, the first pass only counts
+        // (nothing is written), so the storage is allocated once at its
+        // measured size.
+        const bool early = c->list_alloc > 0 && c->list_cap > 0 && c->wq &&
+                           !(c->quad && !c->list_q);
+        int rc = early ? NB_OK : read_counters(c);
         if (rc) return rc;
-        const int64_t G = c->cnt_host[CNT_GROUPS];
-        c->groups_host = G;
-        // With no list storage yet, the first pass only counts (nothing is
-        // written), so the storage is allocated once at its measured size.
         int64_t cap = c->list_cap > 0 ? c->list_cap : 0;
         if (c->list_alloc == 0 && c->cfg.list_capacity <= 0) cap = 0;
-        for (int attempt = 0; attempt < 6; attempt++) {
+        for (int attempt = early ? -1 : 0; attempt < 6; attempt++) {
             const bool counting = cap == 0;
             if (counting) {
                 c->list_cap = 0;
-            } else {
-                rc = ensure_lists(c, G, cap);
+            } else if (attempt >= 0) {
+                rc = ensure_lists(c, c->cnt_host[CNT_GROUPS], cap);
                 if (rc) return rc;
             }
             nb_launch_walk(c);
             if (cudaGetLastError() != cudaSuccess) return NB_ERR_CUDA;
             unsigned bits = 0;
-            rc = sync_read_bits(c, &bits);
+            rc = sync_read_all(c, &bits);
             if (rc) return rc;
+            c->groups_host = c->cnt_host[CNT_GROUPS];
             rc = err_code(bits);
             if (rc != NB_OK && rc != NB_ERR_CAPACITY) break;
             if (rc == NB_OK && !counting) break;
-            rc = read_counters(c);
-            if (rc) return rc;
+            if (rc == NB_ERR_CAPACITY) {
+                rc = uncount(c);
+                if (rc) return rc;
+            }
             if (bits & NB_EF_QUEUE) {   // a frontier outgrew the walk queues
                 const int64_t want = 2 * (c->cnt_host[CNT_QMAX] > c->wq_cap ? c->cnt_host[CNT_QMAX]
                                                                             : c->wq_cap);
                 CK(cudaStreamSynchronize(c->stream));
                 if (!alloc_queues(c, want)) return NB_ERR_NOMEM;
-            } else if (counting || (bits & NB_EF_CAPACITY)) {
+            } else if (c->cnt_host[CNT_LIST_MAX] > cap) {   // a list outgrew its slot
                 if (!counting && c->cfg.list_capacity > 0) return NB_ERR_CAPACITY;
                 const int64_t need = c->cnt_host[CNT_LIST_MAX];
                 cap = ((need + need / 4 + 255) / 256) * 256;
                 if (cap < 256) cap = 256;
-            }
+            } else if (counting) {
+                cap = 256;
+            }   // else the early walk met more groups than the storage holds
             rc = NB_ERR_CAPACITY;
         }
         phase_end(c, tk, NB_PHASE_WALK);
@@ -731,6 +730,7 @@ int nb_forces_fused(nb_ctx *c, float theta, int n_crit, float eps, float *acc, f
         if (!(bits & NB_EF_QUEUE)) break;
         // a frontier outgrew the walk queues: grow them and sum again
         rc = read_counters(c);
+        if (!rc) rc = uncount(c);
         if (rc) return rc;
         const int64_t want = 2 * (c->cnt_host[CNT_QMAX] > c->wq_cap ? c->cnt_host[CNT_QMAX]
                                                                     : c->wq_cap);
@@ -894,6 +894,9 @@ int nb_walk_forces(nb_ctx *c, float theta, int n_crit, float eps, float *acc, fl
     if (bits & (NB_EF_CAPACITY | NB_EF_QUEUE)) {
         // a list outgrew its slot or a frontier the queues: the separate,
         // synchronising walk grows the storage, then the force sum again
+        rc = read_counters(c);
+        if (!rc) rc = uncount(c);
+        if (rc) return rc;
         rc = nb_walk_groups(c, theta, n_crit, nullptr);
         if (rc) return rc;
         return nb_forces(c, eps, acc, pot, precision);
