@@ -342,19 +342,27 @@ class NBody:
         off = torch.empty(n + 1, dtype=torch.int64, device="cuda")
         tot = C.c_int64(0)
         # room for as many as the last search of this context found, and an
-        # eighth more: only a search that finds more (or the first) takes a
-        # call of its own to count
+        # eighth more, where it can be had: only a search that finds more (or
+        # the first) takes a call of its own to count
         cap = getattr(self, "_neigh_cap", 0)
-        idx = torch.empty(cap, dtype=torch.int32, device="cuda")
+        try:
+            idx = torch.empty(cap, dtype=torch.int32, device="cuda")
+        except torch.cuda.OutOfMemoryError:
+            cap, idx = 0, None
         _check(_lib.nb_neighbours(self._h, float(h), int(n_crit), off.data_ptr(),
                                   idx.data_ptr() if cap else None, cap, C.byref(tot)),
                "nb_neighbours")
+        self._neigh_cap = tot.value + tot.value // 8
         if tot.value > cap or cap == 0:
             idx = torch.empty(max(tot.value, 1), dtype=torch.int32, device="cuda")
             _check(_lib.nb_neighbours(self._h, float(h), int(n_crit), off.data_ptr(),
                                       idx.data_ptr(), int(idx.numel()), C.byref(tot)),
                    "nb_neighbours")
-        self._neigh_cap = tot.value + tot.value // 8
+        elif tot.value + tot.value // 3 < cap:
+            # a small answer does not keep the room alive (complete on return,
+            # as the library's writes are)
+            idx = idx[:tot.value].clone()
+            torch.cuda.current_stream().synchronize()
         return off, idx[:tot.value]
 
     def walk_forces(self, theta, n_crit, eps, acc, pot=None, precision="fp32"):
