@@ -300,7 +300,9 @@ int nb_graph_launch(nb_ctx *ctx);
  * independent systems when offsets_dev (device, n_systems + 1 row offsets)
  * is given, as nb_build_tree_batched; one system when it is NULL -- then
  * times `reps` walk + FP32 force passes with CUDA events for every n_crit of
- * the list x force work-item width (32 or 64 targets per warp) x j-tile depth
+ * the list x force work-item width (at most 32 or 64 targets per warp; up to
+ * 1.5M particles the items are no wider than 32 either way, so the two widths
+ * are one configuration, timed once and reported as 64) x j-tile depth
  * (32 or 64 list records staged per tile; items of several source streams
  * stage 64 either way) x force block size (256 or 128
  * threads), keeps the fastest combination in the context (cfg.n_crit and the

@@ -275,8 +275,9 @@ class NBody:
 
     def autotune(self, pos, mass, eps, theta, n_crits=(32, 64, 128, 256, 512), reps=3,
                  offsets=None):
-        """Times walk + FP32 force over n_crit x item rows (1, 2: 32 or 64
-        targets per warp) x j-tile depth (32, 64) x block size (256, 128) and
+        """Times walk + FP32 force over n_crit x item rows (1, 2: at most 32 or
+        64 targets per warp; the same items, timed once and reported as 2, up to
+        1.5M particles) x j-tile depth (32, 64) x block size (256, 128) and
         keeps the fastest.  Returns ({"n_crit", "rows", "tile", "block"},
         {(n_crit, rows, tile, block): ms}); offsets (int64 CUDA tensor of
         n_systems + 1 row offsets) tunes a batch of systems."""

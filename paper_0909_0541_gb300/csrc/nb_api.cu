@@ -1095,8 +1095,15 @@ int nb_autotune(nb_ctx *c, const double *pos, const float *mass, const int64_t *
     const int tiles[2] = {32, 64}, blocks[2] = {256, 128};
     float best = INFINITY;
     int bn = n_crit[0], br = rows0, bt = 32, bb = 256;
+    // where the particle count limits the items to 32 targets or fewer, both
+    // widths form the same items: the wider one is timed for both and kept, so
+    // that a later, larger system is not limited
+    c->item_rows = 1;
+    const int narrow = nb_item_block(c);
+    c->item_rows = 2;
+    const int rows_first = nb_item_block(c) == narrow ? 2 : 1;
     for (int k = 0; k < ncand && rc == NB_OK; k++)
-        for (int rows = 1; rows <= 2 && rc == NB_OK; rows++)
+        for (int rows = rows_first; rows <= 2 && rc == NB_OK; rows++)
             for (int ti = 0; ti < 2 && rc == NB_OK; ti++)
                 for (int bi = 0; bi < 2 && rc == NB_OK; bi++) {
                     c->item_rows = rows;
@@ -1118,7 +1125,8 @@ int nb_autotune(nb_ctx *c, const double *pos, const float *mass, const int64_t *
                     float ms = 0.f;
                     cudaEventElapsedTime(&ms, e0, e1);
                     ms /= reps;
-                    if (ms_out) ms_out[((k * 2 + rows - 1) * 2 + ti) * 2 + bi] = ms;
+                    for (int q = rows_first == 2 ? 1 : rows; ms_out && q <= rows; q++)
+                        ms_out[((k * 2 + q - 1) * 2 + ti) * 2 + bi] = ms;
                     if (ms < best) {
                         best = ms;
                         bn = n_crit[k];

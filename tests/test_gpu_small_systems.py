@@ -71,3 +71,19 @@ def test_items_on_both_sides_of_a_line(oracle_lib, n):
             assert np.array_equal(acc.cpu().numpy(), g["acc"])
             assert np.array_equal(pot.cpu().numpy(), g["pot"])
         ctx.close()
+
+
+@pytest.mark.parametrize("n", [3000, 20000])
+def test_autotuner_times_one_width_where_there_is_one(n):
+    """Up to 1.5M particles both item widths form the same items: one timing,
+    reported for both, and the wider one kept for later builds."""
+    import paper_0909_0541_gb300 as nb
+    ps = nbsynth.plummer(n, 9)
+    dev = torch.device("cuda")
+    ctx = nb.NBody(n)
+    pick, table = ctx.autotune(torch.from_numpy(ps.pos).to(dev), torch.from_numpy(ps.mass).to(dev),
+                               1e-3, 0.7, n_crits=(16, 64, 256), reps=2)
+    ctx.close()
+    assert pick["rows"] == 2
+    for (crit, rows, tile, block), ms in table.items():
+        assert ms > 0 and ms == table[(crit, 3 - rows, tile, block)]
