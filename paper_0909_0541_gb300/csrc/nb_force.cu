@@ -635,8 +635,7 @@ __device__ __forceinline__ double widen(float f)
 // 2^-21.  With e = 1 - r2 y^2 the series 1/sqrt(1 - e) = 1 + e/2 + 3 e^2/8 +
 // O(e^3) leaves (5/16) e^3 < 2^-61 beside the rounding of its last steps.
 // Outside FP32's normal range (and for non-finite r2) the square root and
-// the division; r2 = 0 (a coincident pair without softening) gives 0, so
-// that it contributes nothing.
+// the division.
 __device__ __forceinline__ double judge_rsqrt(double r2)
 {
     const unsigned hi = (unsigned)__double2hiint(r2), lo = (unsigned)__double2loint(r2);
@@ -647,7 +646,7 @@ __device__ __forceinline__ double judge_rsqrt(double r2)
         const double e = __fma_rn(-__dmul_rn(r2, y), y, 1.0);
         return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
     }
-    return r2 == 0.0 ? 0.0 : 1.0 / sqrt(r2);
+    return 1.0 / sqrt(r2);
 }
 
 __global__ void __launch_bounds__(DJ_T)
@@ -682,8 +681,11 @@ k_direct(const double *__restrict__ pos, const float *__restrict__ mass, int64_t
         for (int r = 0; r < DJ_R; r++) {
             const double dx = xj - x[r][0], dy = yj - x[r][1], dz = zj - x[r][2];
             const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __fma_rn(dx, dx, eps2)));
+            // the target itself and a coincident pair without softening are left
+            // out, whatever their coordinates and masses
+            if (j == self[r] || (__double2hiint(r2) | __double2loint(r2)) == 0) continue;
             const double ri = judge_rsqrt(r2);
-            const double mr = (j == self[r] ? 0.0 : mj) * ri;
+            const double mr = mj * ri;
             const double w3 = mr * ri * ri;
             v[r][0] = __fma_rn(w3, dx, v[r][0]);
             v[r][1] = __fma_rn(w3, dy, v[r][1]);

@@ -53,3 +53,38 @@ def test_coincident_points_and_extreme_separations(scale):
     pos[100:110] = pos[5]
     mass = np.full(600, 1e-3, np.float32)
     _check(pos, mass, 0.0, [0, 5, 100, 109, 599])
+
+
+def test_left_out_pairs_are_left_out_whatever_they_hold():
+    """The target itself and coincident pairs (eps = 0) add nothing, also where
+    their mass or a coordinate is not finite: the sums of the other pairs."""
+    import paper_0909_0541_gb300 as nb
+    rng = np.random.default_rng(4)
+    n = 700
+    dev = torch.device("cuda")
+    for case in ("mass", "position"):
+        pos, mass = rng.normal(size=(n, 3)), rng.uniform(0.5, 1.5, n).astype(np.float32) / n
+        i = 10
+        if case == "mass":
+            pos[20:23] = pos[i]
+            mass[20], mass[21], mass[i] = np.inf, np.nan, np.inf
+        else:
+            pos[i, 1] = np.inf
+        a, p = nb.direct_sum(torch.from_numpy(pos).to(dev), torch.from_numpy(mass).to(dev), 0.0,
+                             torch.tensor([i], device=dev))
+        a, p = a.cpu().numpy()[0], p.cpu().numpy()[0]
+        m = mass.astype(np.float64)
+        with np.errstate(all="ignore"):
+            d = pos - pos[i]
+            r2 = (d * d).sum(1)
+            ok = (np.arange(n) != i) & (r2 != 0)
+            ri = 1.0 / np.sqrt(r2[ok])
+            want = ((m[ok] * ri * ri * ri)[:, None] * d[ok]).sum(0)
+            wp = -(m[ok] * ri).sum()
+        # FP64 sums in another order; an infinite position leaves 0 x inf = NaN
+        # along its axis and 0 elsewhere
+        assert np.allclose(a, want, rtol=1e-11, atol=1e-12, equal_nan=True), case
+        assert np.isfinite(wp) and abs(p - wp) <= 1e-12 * abs(wp), case
+    one, _ = nb.direct_sum(torch.full((1, 3), np.inf, dtype=torch.float64, device=dev),
+                           torch.ones(1, device=dev), 0.0)
+    assert torch.equal(one, torch.zeros_like(one))
