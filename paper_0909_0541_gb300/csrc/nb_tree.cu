@@ -1128,9 +1128,11 @@ static void sort_by_system(nb_ctx *c, int64_t n, int packed)
     nb_launch(k_sys_key, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, c->sys_of, n, c->skey,
               c->sval);
     nb_launched(c, "k_sys_key");
+    // two 8-bit digits hold 65,536 systems; beyond, four (the number is even)
+    const int passes = c->nsys > 65536 ? 4 : 2;
     nb_radix_sort_passes(c->skey, c->skey_alt, c->sval, c->sval_alt, c->sort_hist, c->scan_bsum,
-                         n, 2, s);
-    c->launches += 2 * 5;
+                         n, passes, s);
+    c->launches += passes * 4;   // counts, a scan of two launches, scatter
     nb_launch(k_sys_apply, nb_grid(n, 256), 256, 0, nb_queue(c), c->keys, c->idx, c->skey, c->sval,
               n, c->keys_alt, c->idx_alt, c->sys_sorted);
     nb_launched(c, "k_sys_apply");

@@ -2,7 +2,9 @@
 sorted values: one digit up to 256 systems, two beyond, odd sizes, and equal
 keys (coincident particles keep the caller's order).  Every system's slots
 must be the stable key order of its own rows, with the keys that system's
-tree gets when it is built alone.
+tree gets when it is built alone.  The same where index and system do not fit
+32 bits and a second sort orders the systems, by two digits up to 65,536
+systems and by four beyond.
 """
 import numpy as np
 import pytest
@@ -49,3 +51,29 @@ def test_order_is_stable_by_system_and_key(nsys, lo, hi):
         assert np.array_equal(o["keys"], keys[a:b]) and np.array_equal(o["perm"] + a, perm[a:b])
         one.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("nsys,lo,hi", [(33000, 1, 3), (65536, 1, 2), (65537, 1, 2),
+                                        (140000, 1, 2)])
+def test_order_by_a_second_sort(nsys, lo, hi):
+    test_order_is_stable_by_system_and_key(nsys, lo, hi)
+
+
+def test_forces_of_more_systems_than_two_digits_hold():
+    """Pairs: each particle's acceleration is its partner's pull alone."""
+    import paper_0909_0541_gb300 as nb
+    nsys = 70_000
+    pos = nbsynth.uniform_cube(2 * nsys, 5).pos
+    dev = torch.device("cuda")
+    x = torch.from_numpy(pos).to(dev)
+    m = torch.full((2 * nsys,), 0.5, dtype=torch.float32, device=dev)
+    acc = torch.empty((2 * nsys, 3), dtype=torch.float32, device=dev)
+    ctx = nb.NBody(2 * nsys, max_systems=nsys)
+    ctx.build_tree_batched(x, m, torch.arange(0, 2 * nsys + 1, 2, device=dev))
+    ctx.walk_groups(0.6, 8)
+    ctx.forces(0.1, acc)
+    ctx.close()
+    d = pos.reshape(nsys, 2, 3)[:, ::-1].reshape(-1, 3) - pos
+    want = 0.5 * d / ((d * d).sum(1) + 0.01)[:, None] ** 1.5
+    # rsqrt to 1.3e-7, cubed, and a few roundings of 6e-8: below 1e-6
+    assert np.abs(acc.cpu().numpy() - want).max() <= 1e-6 * np.abs(want).max()
