@@ -170,6 +170,7 @@ static void carve_context(nb_ctx *c, Arena &a)
         a.carve(&c->sys_of, N);
         a.carve(&c->sys_sorted, N);
         a.carve(&c->sys_root, c->max_sys);
+        a.carve(&c->sys_off, c->max_sys + 1);
         a.carve(&c->skey, N);
         a.carve(&c->skey_alt, N);
         a.carve(&c->sval, N);
@@ -518,7 +519,6 @@ int nb_build_tree_batched(nb_ctx *c, const double *pos, const float *mass,
     c->has_lists = 0;
     c->n = n;
     c->nsys = nsys;
-    c->sys_off = offsets;
     c->tree_quad = c->quad && c->b_q;
     const int tk = phase_begin(c);
     if (nsys == 1) nb_launch_build(c, pos, mass, n);

@@ -64,6 +64,7 @@ enum {
     CNT_MOM_Q,       // moments work queue head (32-cell chunks)
     CNT_MOM_CHUNKS,  // chunks in the moments work list
     CNT_BBOX_DONE,   // blocks of k_bbox_root that have written their partial box
+    CNT_BAD_OFF,     // a batch's offsets are not 0, ascending, n
     CNT_PP_CUM,      // n_pp over every walk (never reset)
     CNT_PC_CUM,
     CNT_BAD_SITE,    // first failed self-check: site code (never reset)
@@ -147,7 +148,7 @@ struct nb_ctx {
     // system in level order; nsys = 1 for a single system
     int64_t nsys, max_sys;
     int32_t *sys_of, *sys_sorted, *sys_root;
-    const int64_t *sys_off;
+    int64_t *sys_off;   // the batch's offsets, checked (max_sys + 1)
     uint64_t *skey, *skey_alt;
     uint32_t *sval, *sval_alt;
 
@@ -270,7 +271,7 @@ struct nb_ctx {
 void nb_exclusive_scan(nb_ctx *c, const int32_t *in, int32_t *out,
                        int64_t n_max, const long long *n_dev, long long *total_dev);
 void nb_radix_sort(nb_ctx *c, int64_t n);
-bool nb_radix_sort_systems(nb_ctx *c, const int64_t *off, int64_t nsys, int64_t n, int bits);
+bool nb_radix_sort_systems(nb_ctx *c, int64_t nsys, int64_t n, int bits);
 void nb_exclusive_scan_raw(const int32_t *in, int32_t *out, int64_t n_max, int32_t *bsum,
                            cudaStream_t s);
 void nb_radix_sort_raw(uint64_t *keys, uint64_t *keys_alt, uint32_t *idx, uint32_t *idx_alt,

@@ -975,19 +975,40 @@ void nb_launch_build(nb_ctx *c, const double *pos, const float *mass, int64_t n)
 }
 
 // ------------------------------------------------------------ batches
-// system of every particle from the (caller-owned) offsets; checks them
+// check of the caller's offsets: 0, ascending, n
 __global__ void __launch_bounds__(256)
-k_sys_of(const int64_t *__restrict__ off, int64_t nsys, int64_t n, int32_t *__restrict__ sys_of,
-         unsigned *__restrict__ err)
+k_sys_check(const int64_t *__restrict__ off, int64_t nsys, int64_t n, long long *__restrict__ cnt,
+            unsigned *__restrict__ err)
 {
     nb_grid_wait();
-    for (int64_t sy = blockIdx.x; sy < nsys; sy += gridDim.x) {
+    for (int64_t sy = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sy < nsys;
+         sy += (int64_t)gridDim.x * blockDim.x) {
         const int64_t a = off[sy], b = off[sy + 1];
-        if (threadIdx.x == 0 && (!(b > a) || a < 0 || b > n || (sy == 0 && a != 0) ||
-                                 (sy == nsys - 1 && b != n)))
+        if (!(b > a) || (sy == 0 && a != 0) || (sy == nsys - 1 && b != n)) {
             atomicOr(err, NB_EF_BADARG);
-        const int64_t lo = a < 0 ? 0 : a, hi = b > n ? n : b;
-        for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) sys_of[i] = (int32_t)sy;
+            cnt[CNT_BAD_OFF] = 1;
+        }
+    }
+}
+
+// The system of every particle, and the context's copy of the offsets, which
+// the build reads from here on.  Bad offsets (reported by the check) are
+// replaced by one particle per system and the rest for the last one, so that
+// every row has a system and every range lies inside the rows.
+__global__ void __launch_bounds__(256)
+k_sys_of(const int64_t *__restrict__ off, int64_t nsys, int64_t n, int64_t *__restrict__ own,
+         int32_t *__restrict__ sys_of, const long long *__restrict__ cnt)
+{
+    nb_grid_wait();
+    const bool bad = cnt[CNT_BAD_OFF] != 0;
+    for (int64_t sy = blockIdx.x; sy < nsys; sy += gridDim.x) {
+        const int64_t a = bad ? sy : off[sy];
+        const int64_t b = sy == nsys - 1 ? n : bad ? sy + 1 : off[sy + 1];
+        if (threadIdx.x == 0) {
+            own[sy] = a;
+            if (sy == nsys - 1) own[nsys] = n;
+        }
+        for (int64_t i = a + threadIdx.x; i < b; i += blockDim.x) sys_of[i] = (int32_t)sy;
     }
 }
 
@@ -998,7 +1019,7 @@ k_sys_of(const int64_t *__restrict__ off, int64_t nsys, int64_t n, int32_t *__re
 #define RS_SYS_T 1024
 __global__ void __launch_bounds__(RS_SYS_T)
 k_roots_sys(const double *__restrict__ pos, const int64_t *__restrict__ off, int64_t nsys,
-            int64_t n, double *__restrict__ roots, unsigned *__restrict__ err)
+            double *__restrict__ roots, unsigned *__restrict__ err)
 {
     nb_grid_wait();
     const long long FLIP = 0x7fffffffffffffffll;
@@ -1006,9 +1027,7 @@ k_roots_sys(const double *__restrict__ pos, const int64_t *__restrict__ off, int
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long *__restrict__ pb = reinterpret_cast<const long long *>(pos);
     for (int64_t sy = blockIdx.x; sy < nsys; sy += gridDim.x) {
-        int64_t a = off[sy], b = off[sy + 1];
-        a = a < 0 ? 0 : (a > n ? n : a);
-        b = b < a ? a : (b > n ? n : b);
+        const int64_t a = off[sy], b = off[sy + 1];
         long long lo[3], hi[3];
         for (int k = 0; k < 3; k++) { lo[k] = LLONG_MAX; hi[k] = LLONG_MIN; }
         bool bad = false;
@@ -1101,17 +1120,15 @@ k_sys_roots(const int32_t *__restrict__ level_start, const int32_t *__restrict__
         sys_root[sys_sorted[n_first[bfs2pid[b]]]] = b;
 }
 
-// the values' packed systems and indices apart (a system number beyond the
-// batch can only come from offsets that the offset check has reported)
+// the values' packed systems and indices apart
 __global__ void __launch_bounds__(256)
-k_sys_unpack(uint32_t *__restrict__ idx, int64_t n, int bits, int64_t nsys,
-             int32_t *__restrict__ sys_sorted)
+k_sys_unpack(uint32_t *__restrict__ idx, int64_t n, int bits, int32_t *__restrict__ sys_sorted)
 {
     nb_grid_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const uint32_t v = idx[i];
-    sys_sorted[i] = (int32_t)min((int64_t)(v >> bits), nsys - 1);
+    sys_sorted[i] = (int32_t)(v >> bits);
     idx[i] = v & ((1u << bits) - 1u);
 }
 
@@ -1121,7 +1138,7 @@ static void sort_by_system(nb_ctx *c, int64_t n, int packed)
 {
     cudaStream_t s = c->stream;
     if (packed) {
-        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, packed, c->nsys,
+        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, packed,
                   c->sys_sorted);
         nb_launched(c, "k_sys_unpack");
     }
@@ -1146,9 +1163,12 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
     cudaStream_t s = c->stream;
     cudaMemsetAsync(c->cnt, 0, sizeof(long long) * CNT_PP_CUM, s);
     const int gs = (int)(nsys < 65535 ? nsys : 65535);
-    nb_launch(k_sys_of, gs, 256, 0, nb_queue(c), off, nsys, n, c->sys_of, c->err);
+    nb_launch(k_sys_check, nb_grid(nsys, 256, c->num_sms), 256, 0, nb_queue(c), off, nsys, n,
+              c->cnt, c->err);
+    nb_launched(c, "k_sys_check");
+    nb_launch(k_sys_of, gs, 256, 0, nb_queue(c), off, nsys, n, c->sys_off, c->sys_of, c->cnt);
     nb_launched(c, "k_sys_of");
-    nb_launch(k_roots_sys, gs, RS_SYS_T, 0, nb_queue(c), pos, off, nsys, n, c->root, c->err);
+    nb_launch(k_roots_sys, gs, RS_SYS_T, 0, nb_queue(c), pos, c->sys_off, nsys, c->root, c->err);
     nb_launched(c, "k_roots_sys");
     // the system rides in the high bits of the sorted values where both fit
     // 32 bits, and one or two more digits sort by it; else a second sort of
@@ -1161,8 +1181,8 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
               c->idx, c->key_order, pack ? bits : 0);
     nb_launched(c, "k_keys");
     nb_radix_sort(c, n);
-    if (pack && nb_radix_sort_systems(c, off, nsys, n, bits)) {
-        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, bits, nsys,
+    if (pack && nb_radix_sort_systems(c, nsys, n, bits)) {
+        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, bits,
                   c->sys_sorted);
         nb_launched(c, "k_sys_unpack");
     } else {

@@ -77,3 +77,28 @@ def test_forces_of_more_systems_than_two_digits_hold():
     want = 0.5 * d / ((d * d).sum(1) + 0.01)[:, None] ** 1.5
     # rsqrt to 1.3e-7, cubed, and a few roundings of 6e-8: below 1e-6
     assert np.abs(acc.cpu().numpy() - want).max() <= 1e-6 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("bad", [[0, 400, 900], [100, 500, 1000], [500, 1500, 1000],
+                                 [0, 600, 500, 1000], [0, 500, 500, 1000], [0, 900, 800],
+                                 [-5, 500, 1000], [300, 100, 1000], [900, 50, 100],
+                                 [0, 2000, 3000]])
+def test_offsets_that_are_no_partition_are_refused(bad):
+    """Invalid argument, whatever an earlier batch left in the context, and the
+    next batch is sorted as ever."""
+    import paper_0909_0541_gb300 as nb
+    n = 1000
+    dev = torch.device("cuda")
+    x = torch.from_numpy(nbsynth.uniform_cube(n, 3).pos).to(dev)
+    m = torch.full((n,), 1.0 / n, dtype=torch.float32, device=dev)
+    good = torch.tensor([0, 100, 200, 300, 400, 1000], device=dev)
+    ctx = nb.NBody(n, max_systems=5)
+    ctx.build_tree_batched(x, m, good)
+    ref = ctx.copy_tree()
+    with pytest.raises(nb.NBError) as e:
+        ctx.build_tree_batched(x, m, torch.tensor(bad, device=dev))
+    assert e.value.code == -1
+    ctx.build_tree_batched(x, m, good)
+    t = ctx.copy_tree()
+    assert all(np.array_equal(ref[k], t[k]) for k in ("keys", "perm", "first", "count", "com"))
+    ctx.close()
