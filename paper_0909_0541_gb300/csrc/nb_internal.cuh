@@ -271,7 +271,7 @@ struct nb_ctx {
 void nb_exclusive_scan(nb_ctx *c, const int32_t *in, int32_t *out,
                        int64_t n_max, const long long *n_dev, long long *total_dev);
 void nb_radix_sort(nb_ctx *c, int64_t n);
-bool nb_radix_sort_systems(nb_ctx *c, int64_t nsys, int64_t n, int bits);
+void nb_radix_sort_systems(nb_ctx *c, int64_t nsys, int64_t n, int bits);
 void nb_exclusive_scan_raw(const int32_t *in, int32_t *out, int64_t n_max, int32_t *bsum,
                            cudaStream_t s);
 void nb_radix_sort_raw(uint64_t *keys, uint64_t *keys_alt, uint32_t *idx, uint32_t *idx_alt,

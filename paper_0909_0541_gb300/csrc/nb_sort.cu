@@ -487,13 +487,11 @@ k_rs_sys_hist(const int64_t *__restrict__ off, int64_t nsys, uint32_t *__restric
 
 // Sort the key-sorted (c->keys, c->idx) stably by the system number held in
 // the values from bit `bits` on (nsys <= 65536): one or two more single-pass
-// digits.  False if the status words have no room (the caller sorts by other
-// means).  Result in c->keys / c->idx.
-bool nb_radix_sort_systems(nb_ctx *c, int64_t nsys, int64_t n, int bits)
+// digits (the context's status words hold eight).  Result in c->keys / c->idx.
+void nb_radix_sort_systems(nb_ctx *c, int64_t nsys, int64_t n, int bits)
 {
     const int nb = (int)((n + (int64_t)RS_T * RS_I1 - 1) / ((int64_t)RS_T * RS_I1));
     const int64_t words = (int64_t)nb * 256 * 2 + 2 * 256 + 2;
-    if (n >= (int64_t)RS_VAL || words > c->rs_status_len) return false;
     uint32_t *hist = c->rs_status + (int64_t)nb * 256 * 2, *ctr = hist + 2 * 256;
     cudaMemsetAsync(c->rs_status, 0, sizeof(uint32_t) * words, c->stream);
     nb_launch(k_rs_sys_hist, nb_grid(nsys, 256, c->num_sms), 256, 0, nb_queue(c), c->sys_off, nsys,
@@ -507,7 +505,6 @@ bool nb_radix_sort_systems(nb_ctx *c, int64_t nsys, int64_t n, int bits)
         uint64_t *tk = c->keys; c->keys = c->keys_alt; c->keys_alt = tk;
         uint32_t *tv = c->idx; c->idx = c->idx_alt; c->idx_alt = tv;
     }
-    return true;
 }
 
 // ------------------------------------------------------- explicit buffers

@@ -1134,14 +1134,9 @@ k_sys_unpack(uint32_t *__restrict__ idx, int64_t n, int bits, int32_t *__restric
 
 // the key-sorted particles stably by system: a sort of the gathered system
 // numbers, applied to keys and indices
-static void sort_by_system(nb_ctx *c, int64_t n, int packed)
+static void sort_by_system(nb_ctx *c, int64_t n)
 {
     cudaStream_t s = c->stream;
-    if (packed) {
-        nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, packed,
-                  c->sys_sorted);
-        nb_launched(c, "k_sys_unpack");
-    }
     nb_launch(k_sys_key, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, c->sys_of, n, c->skey,
               c->sval);
     nb_launched(c, "k_sys_key");
@@ -1181,12 +1176,13 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
               c->idx, c->key_order, pack ? bits : 0);
     nb_launched(c, "k_keys");
     nb_radix_sort(c, n);
-    if (pack && nb_radix_sort_systems(c, nsys, n, bits)) {
+    if (pack) {
+        nb_radix_sort_systems(c, nsys, n, bits);
         nb_launch(k_sys_unpack, nb_grid(n, 256), 256, 0, nb_queue(c), c->idx, n, bits,
                   c->sys_sorted);
         nb_launched(c, "k_sys_unpack");
     } else {
-        sort_by_system(c, n, pack ? bits : 0);
+        sort_by_system(c, n);
     }
     build_tail(c, pos, mass, n, c->sys_sorted);
     nb_launch(k_sys_roots, nb_grid(nsys, 256, c->num_sms * 4), 256, 0, nb_queue(c), c->level_start,
