@@ -511,7 +511,8 @@ int nb_mlp_grad(const float *params_dev, const float *feat_dev, const float *lab
 /* Adam training (beta 0.9 / 0.999, eps 1e-8, rate lr) over `epochs` passes of
  * n samples in batches of `batch`; order_dev holds epochs x n sample indices
  * (the shuffles, drawn by the caller); adam_m/adam_v start at zero; grad_dev
- * is NB_MLP_NPARAM floats of scratch; loss_per_epoch_dev (nullable) receives
+ * (NB_MLP_NPARAM floats, required) is left as it is: the gradients of a step
+ * stay on the chip; loss_per_epoch_dev (nullable) receives
  * each epoch's summed loss. */
 int nb_mlp_train(float *params_dev, float *adam_m_dev, float *adam_v_dev,
                  const float *feat_dev, const float *labels_dev, int64_t n,
