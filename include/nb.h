@@ -166,7 +166,8 @@ int nb_forces(nb_ctx *ctx, float eps, float *acc_dev, float *pot_dev,
  * the opening angle theta and sums Eq. (gravity) on the fly through a small
  * shared-memory buffer.  acc_dev / pot_dev / precision as nb_forces; the
  * results equal nb_walk_groups + nb_forces bit for bit.  The walk is repeated
- * for each work item (up to 64 targets) of a group.  Afterwards there are no
+ * for each work item (up to 64 targets) of a group, or for each pair of
+ * them.  Afterwards there are no
  * lists to export (nb_forces and nb_copy_lists return NB_ERR_STATE until the
  * next nb_walk_groups).  Interaction counts go to nb_get_stats as for the list
  * path.  Errors: STATE (no tree), INVALID_ARG, CAPACITY (a walk frontier

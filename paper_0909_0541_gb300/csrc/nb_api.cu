@@ -710,6 +710,7 @@ int nb_forces_fused(nb_ctx *c, float theta, int n_crit, float eps, float *acc, f
         return NB_ERR_INVALID_ARG;
     if (!c->has_tree) return NB_ERR_STATE;
     c->has_lists = 0;   // the fused pass leaves no lists behind
+    c->n_crit_cur = n_crit;
     if (c->n == 0) return NB_OK;
     const int tk = phase_begin(c);
     nb_launch_groups(c, theta, n_crit, nullptr);

@@ -16,7 +16,9 @@
 // accelerations equal the list path's bit for bit.
 //
 // An item of a group with several items walks the group again: the walk is
-// repeated per item, and the interaction lists never touch HBM.
+// repeated per item, and the interaction lists never touch HBM.  Two full
+// neighbouring items of 32 or 16 targets can share one walk (E = 2 below, rule
+// at fused_streams).
 #include "nb_force.cuh"
 #include "nb_walk.cuh"
 
@@ -29,14 +31,52 @@
 // fewer registers than the list force kernel has
 static constexpr int FW_UNROLL = 4;
 
+// A lane's sums of one source stream, kept in shared memory while it works on
+// another: the pair sums (FP32), the running sums (compensated; a tile's pair
+// sums are folded into them) or the FP64 sums, 16 words for two targets.
+template <int MODE, int R>
+__device__ __forceinline__ void swap_sums(float4 *park, int lane, Acc<MODE> *A, Sum2 *P)
+{
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        float4 *const pa = park + (2 * r) * NB_WARP + lane, *const pb = pa + NB_WARP;
+        const float4 a = *pa, b = *pb;
+        if constexpr (MODE == MODE_FP32) {
+            *pa = make_float4(P[r].x.x, P[r].x.y, P[r].y.x, P[r].y.y);
+            *pb = make_float4(P[r].z.x, P[r].z.y, P[r].p.x, P[r].p.y);
+            P[r].x = make_float2(a.x, a.y);
+            P[r].y = make_float2(a.z, a.w);
+            P[r].z = make_float2(b.x, b.y);
+            P[r].p = make_float2(b.z, b.w);
+        } else if constexpr (MODE == MODE_COMP) {
+            *pa = make_float4(A[r].x, A[r].y, A[r].z, A[r].p);
+            *pb = make_float4(A[r].cx, A[r].cy, A[r].cz, A[r].cp);
+            A[r].x = a.x; A[r].y = a.y; A[r].z = a.z; A[r].p = a.w;
+            A[r].cx = b.x; A[r].cy = b.y; A[r].cz = b.z; A[r].cp = b.w;
+        } else {
+            double2 *const da = reinterpret_cast<double2 *>(pa);
+            double2 *const db = reinterpret_cast<double2 *>(pb);
+            const double2 u = *da, v = *db;
+            *da = make_double2(A[r].dx, A[r].dy);
+            *db = make_double2(A[r].dz, A[r].dp);
+            A[r].dx = u.x; A[r].dy = u.y; A[r].dz = v.x; A[r].dp = v.y;
+        }
+    }
+}
+
 struct FusedCounts {
     long long pp, pc, tot;
     int32_t mx, qmax;
 };
 
-template <int MODE, bool GUARD, int R, int S>
+// R targets per lane and S source streams, as in the list path.  E = 2: two
+// neighbouring items of R * 16 / S targets, whose lanes would run as 2 S streams,
+// summed by one walk: a lane takes its stream's records of each tile as two
+// streams, one after the other, with the idle stream's sums in `park`.  Each
+// target's sums are the same operations in the same order either way.
+template <int MODE, bool GUARD, int R, int S, int E = 1>
 __device__ __forceinline__ void fused_item(
-    int32_t g, int32_t i0, float4 *buf, int32_t *qa_s, int32_t *qb_s, int32_t *qa, int32_t *qb,
+    int32_t g, int32_t i0, float4 *buf, float4 *park, int32_t *qa_s, int32_t *qb_s, int32_t *qa, int32_t *qb,
     int64_t wq_cap, const nb_wrec *__restrict__ wrec, const int32_t *__restrict__ pid2bfs,
     const int32_t *__restrict__ gnode, const int32_t *__restrict__ gfirst,
     const int32_t *__restrict__ gcount, const float4 *__restrict__ gbox,
@@ -47,9 +87,12 @@ __device__ __forceinline__ void fused_item(
     unsigned *__restrict__ err, unsigned &bad, FusedCounts &fc)
 {
     const unsigned FULL = 0xffffffffu;
+    static_assert(E == 1 || E == 2, "one idle stream");
     constexpr int W = NB_WARP / S;
-    constexpr int FT = item_tile(S, NB_WARP);   // records per summed tile, as the list path
+    constexpr int ST = S * E;   // streams of the list path's item
+    constexpr int FT = item_tile(ST, NB_WARP);   // records per summed tile, as the list path
     constexpr int FK = FT / NB_WARP;
+    constexpr int NL = FT / ST, NM = NB_WARP / ST;   // a stream's records of a tile (list, members)
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int row = lane % W, stream = lane / W;
@@ -79,7 +122,23 @@ __device__ __forceinline__ void fused_item(
         A[r].init();
         P[r].init();
     }
-    // (1) walk, summing every 32 buffered sources
+    int e = 0;   // the stream at work (E = 2)
+    if (E == 2)
+#pragma unroll
+        for (int k = 0; k < 2 * R; k++)
+            park[k * NB_WARP + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    auto sum_list = [&]() {   // the buffered tile
+#pragma unroll 1
+        for (int h = 0; h < E; h++) {
+            if (h > 0) {
+                swap_sums<MODE, R>(park, lane, A, P);
+                e ^= 1;
+            }
+            tile_pass<MODE, GUARD, false, R, NL, FW_UNROLL>(buf, (stream * E + e) * NL, 0, t, kk,
+                                                            eps2, A, P);
+        }
+    };
+    // (1) walk, summing every tile of buffered sources
     const int32_t gpid = gnode[g];
     const int32_t gb = nb_in(gpid >= 0 && gpid < total, cnt, err, SITE_WALK_NODE, gpid)
                            ? pid2bfs[gpid] : -1;
@@ -135,8 +194,7 @@ __device__ __forceinline__ void fused_item(
             nb += __shfl_sync(FULL, incl, 31);
             __syncwarp();
             if (nbuf >= FT) {   // one full tile: sum it, keep the rest
-                tile_pass<MODE, GUARD, false, R, W * FK, FW_UNROLL>(buf, stream * W * FK, 0, t, kk,
-                                                                    eps2, A, P);
+                sum_list();
                 __syncwarp();
                 // move the rest (< 32 records) down by whole record pairs (FT is even)
                 if (lane < ((nbuf - FT + 1) & ~1)) buf[lane] = buf[FT + lane];
@@ -163,8 +221,7 @@ __device__ __forceinline__ void fused_item(
         for (int k = 0; k < FK; k++)
             if (k * NB_WARP + lane >= nbuf) put_rec(buf, k * NB_WARP + lane, pad);
         __syncwarp();
-        tile_pass<MODE, GUARD, false, R, W * FK, FW_UNROLL>(buf, stream * W * FK, 0, t, kk, eps2,
-                                                            A, P);
+        sum_list();
         __syncwarp();
     }
     // (2) the group's own members, j != i
@@ -178,11 +235,38 @@ __device__ __forceinline__ void fused_item(
         }
         put_rec(buf, lane, v);
         __syncwarp();
-        tile_pass<MODE, GUARD, true, R, W>(buf, stream * W, j0 + stream * W, t, kk, eps2, A, P);
+#pragma unroll 1
+        for (int h = 0; h < E; h++) {
+            if (h > 0) {
+                swap_sums<MODE, R>(park, lane, A, P);
+                e ^= 1;
+            }
+            const int b = (stream * E + e) * NM;
+            tile_pass<MODE, GUARD, true, R, NM>(buf, b, j0 + b, t, kk, eps2, A, P);
+        }
         __syncwarp();
     }
 #pragma unroll
     for (int r = 0; r < R; r++) pair_fold<MODE>(A[r], P[r]);
+    if constexpr (E == 2) {   // the sum of the two streams (as stream_sum over the lanes)
+        Acc<MODE> B[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) B[r] = A[r];
+        swap_sums<MODE, R>(park, lane, A, P);
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+            pair_fold<MODE>(A[r], P[r]);
+            if constexpr (MODE == MODE_F64) {
+                A[r].dx += B[r].dx; A[r].dy += B[r].dy; A[r].dz += B[r].dz; A[r].dp += B[r].dp;
+            } else {
+                A[r].x += B[r].x; A[r].y += B[r].y; A[r].z += B[r].z; A[r].p += B[r].p;
+                if constexpr (MODE == MODE_COMP) {
+                    A[r].cx += B[r].cx; A[r].cy += B[r].cy;
+                    A[r].cz += B[r].cz; A[r].cp += B[r].cp;
+                }
+            }
+        }
+    }
     if (lane == 0) {   // interaction counts of this item's targets
         const int32_t mi = ng - i0 < R * W ? ng - i0 : R * W;
         fc.pp += (long long)mi * (len - ncell) + (long long)mi * (ng - 1);
@@ -219,7 +303,8 @@ __device__ __forceinline__ void fused_item(
     }
 }
 
-template <int MODE, bool GUARD>
+// ST > 0: items of 64 / ST targets, of which full neighbours share a walk
+template <int MODE, bool GUARD, int ST>
 __global__ void __launch_bounds__(FW_T)
 k_walk_force(const int32_t *__restrict__ items, const nb_wrec *__restrict__ wrec,
              const int32_t *__restrict__ pid2bfs, const int32_t *__restrict__ gnode,
@@ -233,6 +318,7 @@ k_walk_force(const int32_t *__restrict__ items, const nb_wrec *__restrict__ wrec
 {
     nb_grid_wait();
     __shared__ float4 bufs[FW_WARPS][FW_BUF];
+    __shared__ float4 parks[ST ? FW_WARPS : 1][ST ? 4 * NB_WARP : 1];
     __shared__ int32_t sq[FW_WARPS][2 * WQ_SMEM];
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -259,12 +345,24 @@ k_walk_force(const int32_t *__restrict__ items, const nb_wrec *__restrict__ wrec
             if (lane == 0) nb_bad(cnt, err, SITE_FORCE, g);
             continue;
         }
-#define NB_FUSED_ITEM(R, S)                                                                    \
-    fused_item<MODE, GUARD, R, S>(g, i0, bufs[w], sq[w], sq[w] + WQ_SMEM, qa, qb, wq_cap, wrec, \
-                                  pid2bfs, gnode, gfirst, gcount, gbox, p_hi, p_lo, perm, total,  \
-                                  n, eps2, sys_sorted, sys_root, acc, pot, cnt, err, bad, fc)
+#define NB_FUSED_ARGS                                                                          \
+    g, i0, bufs[w], parks[ST ? w : 0], sq[w], sq[w] + WQ_SMEM, qa, qb, wq_cap, wrec, pid2bfs,  \
+        gnode, gfirst, gcount, gbox, p_hi, p_lo, perm, total, n, eps2, sys_sorted, sys_root,   \
+        acc, pot, cnt, err, bad, fc
+#define NB_FUSED_ITEM(R, S) fused_item<MODE, GUARD, R, S>(NB_FUSED_ARGS)
+        if constexpr (ST > 0) {
+            constexpr int32_t T = 64 / ST;
+            const int32_t left = gcount[g] - i0;
+            if (left >= T && ((i0 / T) & 1)) continue;   // summed with the item before it
+            if (left >= 2 * T) {
+                fused_item<MODE, GUARD, 2, ST / 2, 2>(NB_FUSED_ARGS);
+                if (bad) break;
+                continue;
+            }
+        }
         NB_ITEM_SHAPES(word, NB_FUSED_ITEM);
 #undef NB_FUSED_ITEM
+#undef NB_FUSED_ARGS
         if (bad) break;
     }
     if (lane == 0) {
@@ -279,23 +377,54 @@ k_walk_force(const int32_t *__restrict__ items, const nb_wrec *__restrict__ wrec
     }
 }
 
-template <int MODE, bool GUARD>
-static void launch_fused(nb_ctx *c, float eps2, float *acc, float *pot)
+// Source streams of the items whose full neighbours share a walk (2 for items
+// of 32 targets, 4 for 16), or 0: every item walks for itself.  Sharing saves
+// walks and halves the units of work, so it pays with several items for every
+// resident warp (8 on an SM, at 230 to 250 registers a thread) and several items
+// in a group.  Measured, us, items that walk for themselves / sharing / the pass
+// when its items held 64 targets: 1M Plummer, groups of 512: 5414 / 4201 / 4116;
+// 500,000 halos, 256: 1762 / 1676 / 1642; 150,000 Plummer, 512: 869 / 763 / 753;
+// 65,536 Plummer, 1024: 549 / 469 / 472; 32,768 Plummer, 512: 349 / 264 / 335.
+// Below the line: 65,536 halos, 128: 275 / 316 / 322; 40,000 halos, 1024: 238 /
+// 309 / 312; 16,384 halos, 256: 141 / 161 / 210.  Just below it walking alone is
+// the slowest of the three in places (40,000 Plummer, 256: 288 / 257 / 269).
+static int fused_streams(const nb_ctx *c)
+{
+    const int ib = nb_item_block(c);
+    if (ib != 32 && ib != 16) return 0;
+    const double waves = (double)c->n / ib / (8.0 * c->num_sms);   // items per resident warp
+    const bool share = waves >= 1.25 && c->n_crit_cur >= 128 && waves * c->n_crit_cur >= 20.0 * ib;
+    return share ? 64 / ib : 0;
+}
+
+template <int MODE, bool GUARD, int ST>
+static void launch_fused_t(nb_ctx *c, float eps2, float *acc, float *pot)
 {
     static int blocks = 0;
     if (blocks == 0) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_walk_force<MODE, GUARD>, FW_T, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_walk_force<MODE, GUARD, ST>, FW_T,
+                                                      0);
         if (blocks < 1) blocks = 1;
     }
     // one pair of frontier queues per warp: no more warps than the queues hold
     int grid = c->num_sms * blocks;
     if ((int64_t)grid * FW_WARPS > c->walk_warps) grid = c->walk_warps / FW_WARPS;
     if (grid < 1) grid = 1;
-    nb_launch(k_walk_force<MODE, GUARD>, grid, FW_T, 0, nb_queue(c), c->items, c->wrec, c->pid2bfs,
+    nb_launch(k_walk_force<MODE, GUARD, ST>, grid, FW_T, 0, nb_queue(c), c->items, c->wrec, c->pid2bfs,
               c->gnode, c->gfirst, c->gcount, c->gbox, c->p_hi, c->p_lo, c->perm, c->cnt, c->wq,
               c->wq_cap, c->err, eps2, acc, pot, c->n, c->max_items,
               c->nsys > 1 ? c->sys_sorted : nullptr, c->nsys > 1 ? c->sys_root : nullptr);
     nb_launched(c, "k_walk_force");
+}
+
+template <int MODE, bool GUARD>
+static void launch_fused(nb_ctx *c, float eps2, float *acc, float *pot)
+{
+    switch (fused_streams(c)) {
+    case 2: launch_fused_t<MODE, GUARD, 2>(c, eps2, acc, pot); break;
+    case 4: launch_fused_t<MODE, GUARD, 4>(c, eps2, acc, pot); break;
+    default: launch_fused_t<MODE, GUARD, 0>(c, eps2, acc, pot);
+    }
 }
 
 void nb_launch_fused(nb_ctx *c, float eps, float *acc, float *pot, int precision)
