@@ -613,8 +613,12 @@ void nb_launch_walk_force(nb_ctx *c, float eps, float *acc, float *pot, int prec
 // A block takes DJ_R targets (two share a source's loads: 71.5 against 73.6
 // ms with one, 98 with four, whose registers leave too few warps; warps of 8
 // or 32 targets reading the same source: 76 and 87 ms) and its threads stride
-// over the sources.  With few targets the blocks of a cluster share the
-// sources.  The threads' sums are added by shuffles, then over the warps and
+// over the sources.  Up to one target per SM a block takes one, which halves
+// its share of the pipe and doubles the warps: 1 target, 1000 sources 18.5 ->
+// 10.3 us, 1500 24.6 -> 13.7, 200,000 262 -> 137 (with one block per target and
+// the square root and division 16.4, 17.4 and 1600); 152 targets, 20,000 152 ->
+// 139; 100 targets, 200,000 776 -> 798.  With few targets the blocks of a cluster
+// share the sources.  The threads' sums are added by shuffles, then over the warps and
 // the cluster's blocks in a fixed order: the result does not depend on
 // timing, and no workspace is needed.
 #define DJ_T 256
@@ -649,22 +653,23 @@ __device__ __forceinline__ double judge_rsqrt(double r2)
     return 1.0 / sqrt(r2);
 }
 
+template <int R>
 __global__ void __launch_bounds__(DJ_T)
 k_direct(const double *__restrict__ pos, const float *__restrict__ mass, int64_t n,
          double eps2, const int64_t *__restrict__ targets, int64_t first, int64_t nt,
          double *__restrict__ acc, double *__restrict__ pot)
 {
     constexpr int WARPS = DJ_T / NB_WARP;
-    __shared__ double part[WARPS][DJ_R][4];
-    __shared__ double sum[DJ_R][4];
+    __shared__ double part[WARPS][R][4];
+    __shared__ double sum[R][4];
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t t0 = first + (int64_t)(blockIdx.x / C) * DJ_R;
-    double x[DJ_R][3], v[DJ_R][4];
-    int64_t self[DJ_R];
+    const int64_t t0 = first + (int64_t)(blockIdx.x / C) * R;
+    double x[R][3], v[R][4];
+    int64_t self[R];
 #pragma unroll
-    for (int r = 0; r < DJ_R; r++) {
+    for (int r = 0; r < R; r++) {
         const int64_t t = t0 + r < nt ? t0 + r : nt - 1;
         self[r] = targets ? targets[t] : t;
 #pragma unroll
@@ -678,7 +683,7 @@ k_direct(const double *__restrict__ pos, const float *__restrict__ mass, int64_t
         const double xj = pos[3 * j], yj = pos[3 * j + 1], zj = pos[3 * j + 2];
         const double mj = widen(mass[j]);
 #pragma unroll
-        for (int r = 0; r < DJ_R; r++) {
+        for (int r = 0; r < R; r++) {
             const double dx = xj - x[r][0], dy = yj - x[r][1], dz = zj - x[r][2];
             const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __fma_rn(dx, dx, eps2)));
             // the target itself and a coincident pair without softening are left
@@ -696,23 +701,23 @@ k_direct(const double *__restrict__ pos, const float *__restrict__ mass, int64_t
 #pragma unroll
     for (int o = 1; o < NB_WARP; o <<= 1)
 #pragma unroll
-        for (int r = 0; r < DJ_R; r++)
+        for (int r = 0; r < R; r++)
 #pragma unroll
             for (int k = 0; k < 4; k++) v[r][k] += __shfl_xor_sync(0xffffffffu, v[r][k], o);
     if (lane == 0)
 #pragma unroll
-        for (int r = 0; r < DJ_R; r++)
+        for (int r = 0; r < R; r++)
 #pragma unroll
             for (int k = 0; k < 4; k++) part[w][r][k] = v[r][k];
     __syncthreads();
     const int r = threadIdx.x >> 2, k = threadIdx.x & 3;
-    if (r < DJ_R) {
+    if (r < R) {
         double s = part[0][r][k];
         for (int p = 1; p < WARPS; p++) s += part[p][r][k];
         sum[r][k] = s;
     }
     cl.sync();
-    if (rank == 0 && r < DJ_R && t0 + r < nt) {
+    if (rank == 0 && r < R && t0 + r < nt) {
         double s = sum[r][k];
         for (int p = 1; p < C; p++) s += *cl.map_shared_rank(&sum[r][k], p);
         if (k < 3) acc[3 * (t0 + r) + k] = s;
@@ -734,7 +739,8 @@ int nb_launch_direct(const double *pos, const float *mass, int64_t n, double eps
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t tb = (nt + DJ_R - 1) / DJ_R;
+    const int R = nt <= sms ? 1 : DJ_R;
+    const int64_t tb = (nt + R - 1) / R;
     int C = 1;
     while (C < 8 && tb * C < 24 * (int64_t)sms && n >= 2048 * (int64_t)(2 * C)) C *= 2;
     const int64_t max_tb = (int64_t)INT32_MAX / C;
@@ -750,9 +756,9 @@ int nb_launch_direct(const double *pos, const float *mass, int64_t n, double eps
         at[0].val.clusterDim.x = C;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, k_direct, pos, mass, n, eps * eps, targets, done * DJ_R, nt,
-                               acc, pot) != cudaSuccess)
+        cfg.numAttrs = C > 1 ? 1 : 0;
+        if (cudaLaunchKernelEx(&cfg, R == 1 ? k_direct<1> : k_direct<DJ_R>, pos, mass, n, eps * eps,
+                               targets, done * R, nt, acc, pot) != cudaSuccess)
             return -1;
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;

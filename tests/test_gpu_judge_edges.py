@@ -46,6 +46,16 @@ def test_splits(n, nt):
     _check(pos, mass, 1.0 / 64, t)
 
 
+@pytest.mark.parametrize("more", [-1, 0, 1, 2])
+@pytest.mark.parametrize("n", [300, 5000])
+def test_one_and_two_targets_per_block(n, more):
+    """Either side of one target per SM, where a block takes a second one."""
+    rng = np.random.default_rng(n + more)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    mass = rng.uniform(0.5, 1.5, n).astype(np.float32) / n
+    _check(rng.normal(size=(n, 3)), mass, 1.0 / 64, rng.integers(0, n, sms + more))
+
+
 @pytest.mark.parametrize("scale", [1.0, 1e-95, 1e-19, 1e18, 1e100, 1e148, 1e160])
 def test_coincident_points_and_extreme_separations(scale):
     rng = np.random.default_rng(9)
