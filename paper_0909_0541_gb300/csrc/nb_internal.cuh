@@ -402,12 +402,15 @@ static __device__ __forceinline__ int32_t nb_block_scan256(int32_t v, int32_t *t
 // is a chain of about 40 dependent kernels, and below some 100,000 particles
 // the gaps between them were a third of its time (build, walk and force with
 // plain launches and with these: 355 -> 274 us at 1000 particles, 513 -> 427
-// at 16,384, 1343 -> 1276 at 500,000, 2593 -> 2491 at 2.1M).  A captured
-// graph's gaps are shorter (a step of 16,384: 389 -> 370 us, of 65,536 533 ->
-// 494, of 500,000 1222 -> 1227), and in large steps the early blocks cost more
-// than the gaps (1.93M particles 4.27 -> 4.47 ms; 7.66M in 512 systems 10.53
-// -> 10.83).  So launches overlap up to NB_OVERLAP_MAX_N particles, in a
-// capture up to NB_OVERLAP_GRAPH_MAX_N.  Every kernel of the chain calls
+// at 16,384).  Eager calls gain 40 to 70 us at every size measured (1296 -> 1228
+// us at 500,000 particles, 4084 -> 4020 at 2.0M, 4901 -> 4832 at 2.4M, 5200 ->
+// 5140 at 2.6M, 5933 -> 5882 at 3.0M, 7735 -> 7672 at 4.0M, 15.00 -> 14.96 ms at
+// 7.66M): up to NB_OVERLAP_MAX_N particles more than one per cent, beyond it
+// less, and launches stay plain.  A captured graph's gaps are shorter (a step of
+// 16,384: 389 -> 370 us, of 65,536 533 -> 494, of 500,000 1222 -> 1227), and in
+// large steps the early blocks cost more than the gaps (1.93M particles 4.27 ->
+// 4.47 ms; 7.66M in 512 systems 10.53 -> 10.83), so in a capture launches
+// overlap up to NB_OVERLAP_GRAPH_MAX_N.  Every kernel of the chain calls
 // nb_grid_wait first, in every thread: what comes before it is then complete,
 // and through it all earlier launches.
 __device__ __forceinline__ void nb_grid_wait()

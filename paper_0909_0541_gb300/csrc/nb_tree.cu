@@ -1165,9 +1165,12 @@ void nb_launch_build_batched(nb_ctx *c, const double *pos, const float *mass, in
     nb_launched(c, "k_sys_of");
     nb_launch(k_roots_sys, gs, RS_SYS_T, 0, nb_queue(c), pos, c->sys_off, nsys, c->root, c->err);
     nb_launched(c, "k_roots_sys");
-    // the system rides in the high bits of the sorted values where both fit
+    // The system rides in the high bits of the sorted values where both fit
     // 32 bits, and one or two more digits sort by it; else a second sort of
-    // the gathered system numbers
+    // the gathered system numbers.  7.66M particles in 512 systems fill the 32
+    // bits: two captured steps of them take 20.56 ms so and 20.95 with the
+    // second sort, which larger batches take (8.4M particles in more than 256
+    // systems).
     int bits = 1, sbits = 1;
     while ((n - 1) >> bits) bits++;
     while ((nsys - 1) >> sbits) sbits++;
@@ -1876,10 +1879,12 @@ static void launch_topology_small(nb_ctx *c, int64_t n)
 // 142 / 94 / 67 / 55; 65,536 halos 224 / 142 / 89 / 76; 150,000 halos 214 /
 // 144 / 116 / 154; 500,000 halos 571 / 481 / 463 / 670 (quadrupole 1350 / 1155
 // / 1275 / 1451); 1M halos 1018 / 963 / 980 / 1452; 2M halos 1022 / 1022 /
-// 1065 / 1565.  The fused pass repeats its walk for every item, so 16 and 8
-// are taken only where it gains as well or loses little (16,384 halos 162 /
-// 135 / 122 / 167; 65,536 halos 270 / 234 / 282 / 425).  The choice depends on
-// the particle count alone: every path sums the same items in the same order.
+// 1065 / 1565.  The fused pass repeats its walk for every item (for every pair
+// of them where groups are large, nb_fused.cu), so 16 and 8 are taken only where
+// it gains as well or loses little (each item walking alone: 16,384 halos 162 /
+// 135 / 122 / 167; 65,536 halos 270 / 234 / 282 / 425); the list path alone would
+// take 8 at 16,384 and 16 up to 150,000.  The choice depends on the particle
+// count alone: every path sums the same items in the same order.
 int nb_item_block(const nb_ctx *c)
 {
     const int rows = c->item_rows * NB_WARP;
